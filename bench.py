@@ -333,7 +333,7 @@ def main():
     clocks = sampler.stop(t_wall0, t_wall1)
     rows_per_step = w.B * w.rows_target
     value, ms_step = replicas.whole_job_rate(rows_per_step, args.steps, ev0.elapsed_time(ev1), dist, "cuda")
-    launched = "ersd_gsd_verify: statistics, scan, race and merge kernels" if args.entry == "gsd" else binding.ersd_last_launch()
+    launched = "ersd_gsd_verify: gsd_stats_kernel, gsd_race_kernel" if args.entry == "gsd" else binding.ersd_last_launch()
     mean_accept = float(accept.float().mean().item())
 
     # ---- roofline of the one kernel a step launches
@@ -411,7 +411,7 @@ def main():
             "config": dict(workload_config(w, l2_note(alg_bytes, len(sets))),
                            entry={"tokens": "ersd_verify_tokens", "gsd": "ersd_gsd_verify"}.get(
                                args.entry, "ersd_verify_tree" if w.is_tree else "ersd_verify")),
-            "clocks": clocks, "e2e": e2e, "gpu_launches": args.steps * (4 if args.entry == "gsd" else 1),
+            "clocks": clocks, "e2e": e2e, "gpu_launches": args.steps * (2 if args.entry == "gsd" else 1),
             "roofline": roofline,
             "cpu_baseline": cpu, "parity_on_cpu_sample": parity, "mean_accept_len": mean_accept}))
     if dist is not None:

@@ -228,9 +228,10 @@ int ersd_verify_tokens(const void* target_logits, const int32_t* draft_tokens, e
  * the token that ends the call is the winner of an exponential race over the
  * residual (or target) law, argmin_i e_i / w_i, with e_i from counter
  * (i >> 2, position, sequence id, 2) -- both independent of the drafting races
- * (last counter word 0), as Algorithm 1 requires.  All arithmetic is double
- * precision; the call is four small launches, not the single streaming launch
- * of ersd_verify.
+ * (last counter word 0), as Algorithm 1 requires.  Every decision is the one that
+ * double precision takes: single precision with proven error bounds decides where
+ * they allow it, double precision the rest.  The call is two launches, not the
+ * single streaming launch of ersd_verify.
  *   target_logits device [B, k+1, V]   draft_logits device [B, k, V]
  *   draft_tokens  device [B, k] int32  out_tokens device [B, k+1] int32 (-1 padded)
  *   out_accept_len device [B] int32

@@ -11,6 +11,8 @@
 // last block of a sequence turns the winners into the accepted prefix
 // (sequence scan or tree walk) in the same launch.
 #include <cuda_runtime.h>
+#include <math.h>
+#include <stddef.h>
 #include <stdint.h>
 #include <stdio.h>
 #include <string.h>
@@ -52,6 +54,21 @@ struct TreeDesc {  // draft tree of one call, passed by value in kernel paramete
   uint8_t nchild[ERSD_MAX_ROWS];
   uint8_t order[ERSD_MAX_ROWS];  // launch order of rows: rows with a draft row first
 };
+
+// The 16 bytes that start `a` bytes (0 < a < 16) into the 32 bytes lo, hi.  (`a` is the same for a
+// whole row: the switch does not diverge.)
+__device__ __forceinline__ uint4 bytes_from(const uint4& lo, const uint4& hi, unsigned a) {
+  uint32_t w[5];
+  switch (a >> 2) {
+    case 0: w[0] = lo.x; w[1] = lo.y; w[2] = lo.z; w[3] = lo.w; w[4] = hi.x; break;
+    case 1: w[0] = lo.y; w[1] = lo.z; w[2] = lo.w; w[3] = hi.x; w[4] = hi.y; break;
+    case 2: w[0] = lo.z; w[1] = lo.w; w[2] = hi.x; w[3] = hi.y; w[4] = hi.z; break;
+    default: w[0] = lo.w; w[1] = hi.x; w[2] = hi.y; w[3] = hi.z; w[4] = hi.w; break;
+  }
+  const unsigned bits = (a & 3) * 8;
+  return make_uint4(__funnelshift_r(w[0], w[1], bits), __funnelshift_r(w[1], w[2], bits),
+                    __funnelshift_r(w[2], w[3], bits), __funnelshift_r(w[3], w[4], bits));
+}
 
 enum Mode { kSample = 0, kVerify = 1 };
 
@@ -719,12 +736,6 @@ static int noalloc_scratch(void** out) {
 // ---------------------------------------------------------------------------------------------
 #include "ersd_gsd.inc"
 
-// Scratch of a sequence-GSD call, carved from the front of the workspace: softmax statistics
-// [B, 2k+1, 2] doubles, partial winners [B, S] (double, int), first rejections [B].
-static size_t gsd_scratch_bytes(int64_t B, int64_t k, int64_t S) {
-  return (size_t)(B * ((2 * k + 1) * 16 + S * 16 + 8));
-}
-
 static int gsd_check(const void* target, const void* draft, const int32_t* draft_tok, int dt,
                      const uint64_t* seeds, int B, int rows, int V, float T, const void* out_tokens,
                      const void* out_accept_len, bool need_draft) {
@@ -737,6 +748,19 @@ static int gsd_check(const void* target, const void* draft, const int32_t* draft
     if (((uintptr_t)draft & (elem_size(dt) - 1)) != 0 || ((uintptr_t)draft_tok & 3) != 0) return ERSD_EALIGN;
   }
   return ERSD_OK;
+}
+
+// Length of a slice (a multiple of eight) of rows of V logits, and their number: up to `slices` in
+// all, but none shorter than one group of eight per thread.
+static int gsd_slice(int V, int64_t rows, int64_t slices, int threads, int* S) {
+  int64_t n = slices / rows;
+  const int64_t most = ((int64_t)V + 8 * threads - 1) / (8 * threads);
+  if (n > most) n = most;
+  if (n > kGsdSlices) n = kGsdSlices;
+  if (n < 1) n = 1;
+  const int len = (int)((((int64_t)V + n - 1) / n + 7) / 8 * 8);
+  *S = (int)(((int64_t)V + len - 1) / len);
+  return len;
 }
 
 static void gsd_fill(GsdParams& g, const ersd_opts& o, const void* target, const void* draft,
@@ -935,41 +959,28 @@ int ersd_gsd_verify(const void* target_logits, const void* draft_logits, const i
   gsd_fill(g, o, target_logits, draft_logits, draft_tokens, seeds, B, k, V, T, k + 1, k, out_tokens,
            out_accept_len);
   if (g.ld_t < V || g.ld_d < V) return ERSD_EINVAL;
-  // slices of the final race: about two blocks per multiprocessor in all, at least 4096 tokens each
-  int S = (2 * sm_count() + B - 1) / B;
-  if (S > (V + 4095) / 4096) S = (V + 4095) / 4096;
-  if (S > 64) S = 64;
-  if (S < 1) S = 1;
-  g.S = S;
-  const size_t need = gsd_scratch_bytes(B, k, S);  // (never more than ersd_workspace_bytes(B, k + 1))
+  // Sums: about 64 warps per multiprocessor in all, two waves of the 32 that are resident (32 or 128
+  // per multiprocessor: 1 and 4 % slower at 64 sequences of 128256 logits).  Race: one wave of three
+  // blocks per multiprocessor, because a block begins with the ratio tests.
+  g.slice1 = gsd_slice(V, (int64_t)B * (2 * k + 1), 64 * (int64_t)sm_count(), 128, &g.S1);
+  g.slice = gsd_slice(V, B, 3 * (int64_t)sm_count(), kGsdThreads, &g.S);
+  g.sum_err = (float)(4.76837158203125e-7 + 2.384185791015625e-7 * (log2((double)V) + 32.0));
   void* ws = nullptr;
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   st = get_workspace(o, workspace_bytes(B, k + 1), &ws, stream);
   if (st != ERSD_OK) return st;
-  char* w = (char*)ws;
-  g.stats = (double*)w;
-  w += (size_t)B * (2 * k + 1) * 16;
-  g.part_t = (double*)w;
-  w += (size_t)B * S * 8;
-  g.part_i = (int*)w;
-  w += (size_t)B * S * 4;
-  g.jstar = (int*)w;
-  const dim3 rows_grid((unsigned)(2 * k + 1), (unsigned)B), race_grid((unsigned)S, (unsigned)B);
-  const unsigned seq_blocks = (unsigned)((B + 127) / 128);
+  g.slots = (Slot*)ws;
+  const int per_block = kGsdStatsThreads / 32;  // slices of a block of the sums
+  const dim3 sums_grid((unsigned)(2 * k + 1), (unsigned)B, (unsigned)((g.S1 + per_block - 1) / per_block));
+  const dim3 race_grid((unsigned)g.S, (unsigned)B);
   if (dt == ERSD_BF16) {
-    gsd_stats_kernel<ERSD_BF16><<<rows_grid, kGsdThreads, 0, stream>>>(g);
-    gsd_scan_kernel<ERSD_BF16><<<seq_blocks, 128, 0, stream>>>(g);
+    gsd_stats_kernel<ERSD_BF16><<<sums_grid, kGsdStatsThreads, 0, stream>>>(g);
     gsd_race_kernel<ERSD_BF16><<<race_grid, kGsdThreads, 0, stream>>>(g);
   } else {
-    gsd_stats_kernel<ERSD_F32><<<rows_grid, kGsdThreads, 0, stream>>>(g);
-    gsd_scan_kernel<ERSD_F32><<<seq_blocks, 128, 0, stream>>>(g);
+    gsd_stats_kernel<ERSD_F32><<<sums_grid, kGsdStatsThreads, 0, stream>>>(g);
     gsd_race_kernel<ERSD_F32><<<race_grid, kGsdThreads, 0, stream>>>(g);
   }
-  gsd_finish_kernel<<<seq_blocks, 128, 0, stream>>>(g);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(e);
-  // the workspace's resting state is all zero (the race kernels' arrival counters count on it)
-  e = cudaMemsetAsync(ws, 0, need, stream);
+  const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? ERSD_OK : cuda_fail(e);
 }
 

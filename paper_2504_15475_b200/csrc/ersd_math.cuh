@@ -48,19 +48,19 @@ ERSD_HD void philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, u
   out[3] = c3;
 }
 
-// Philox4x32-10 for one race: the counter is (c0, position, sequence id, 0) with only c0
-// varying along a row, so everything that does not depend on c0 is folded once per row:
+// Philox4x32-10 for one race: the counter is (c0, position, sequence id, stream) with only c0
+// varying along a row (stream 0: the races of the method; the comparison verifier draws from others), so everything that does not depend on c0 is folded once per row:
 // round 1 needs one product (the other multiplies the sequence id), round 2 one product
 // (its c0 is a row constant), and three of the key/word xors collapse into constants.
 // 18 wide multiplies and 19 xors per call instead of 20 and 20.
 struct PhiloxRow {
-  uint32_t r1_k1;        // round 1: c2' = hi(M0*c0) ^ r1_k1            (c3 = 0)
+  uint32_t r1_k1;        // round 1: c2' = hi(M0*c0) ^ r1_k1            (r1_k1 = stream ^ k1[0])
   uint32_t r2_a;         // round 2: c0' = hi(M1*c2) ^ r2_a             (r2_a = lo(M1*seq) ^ k0[1])
   uint32_t r2_b;         // round 2: c2' = c3 ^ r2_b                    (r2_b = hi(M0*A0) ^ k1[1])
   uint32_t r3_b;         // round 3: c2' = hi(M0*c0) ^ r3_b             (r3_b = lo(M0*A0) ^ k1[2])
   uint32_t k0[10], k1[10];  // round keys (entries 2.. / 3.. are used)
 
-  ERSD_HD void init(uint64_t seed, uint32_t seq_id, uint32_t position) {
+  ERSD_HD void init(uint64_t seed, uint32_t seq_id, uint32_t position, uint32_t stream = 0) {
     uint32_t a = (uint32_t)seed, b = (uint32_t)(seed >> 32);
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
@@ -73,7 +73,7 @@ struct PhiloxRow {
     mulhilo(kPhiloxM1, seq_id, hi1, lo1);
     const uint32_t A0 = hi1 ^ position ^ k0[0];  // c0 after round 1
     mulhilo(kPhiloxM0, A0, H0, L0);
-    r1_k1 = k1[0];
+    r1_k1 = stream ^ k1[0];
     r2_a = lo1 ^ k0[1];
     r2_b = H0 ^ k1[1];
     r3_b = L0 ^ k1[2];

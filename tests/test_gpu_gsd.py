@@ -161,3 +161,85 @@ def test_gsd_and_ersd_acceptance_on_the_same_rows(ersd):
     sd = math.sqrt((a_gsd * (1 - a_gsd)).sum())
     assert abs(got_g - a_gsd.sum()) < 4.5 * sd, (got_g, a_gsd.sum())
     assert d_hm.sum() - 4.5 * sd <= got_e <= a_gsd.sum() + 4.5 * sd, (got_e, d_hm.sum(), a_gsd.sum())
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("V", [1, 7, 8, 9, 1023, 2049, 4099, 40001])
+def test_sequence_gsd_rows_of_any_length(ersd, V, dtype):
+    """Slices of less than one group, ragged ends, rows on every 16-byte offset, NaN and infinite logits."""
+    w = wl.Workload("gsdlen", B=9, k=3, V=V, dtype=dtype, sigma=0.7, T=0.8, config_id=51)
+    inp = wl.make_inputs(w)
+    tok = draft_tokens(ersd, inp["draft"].cuda(), inp["seeds"].cuda(), inp["T"])[..., 0].contiguous()
+    if V > 8:
+        inp["target"][0, :, 1::3] = float("nan")
+        inp["draft"][1, :, 2::3] = float("nan")
+        inp["target"][2, :, V // 2:] = float("-inf")
+        inp["draft"][3, :, : V // 2] = float("-inf")
+        inp["target"][4, 1] = float("-inf")                     # a law without support
+    out = torch.full((w.B, w.k + 1), -9, dtype=torch.int32, device="cuda")
+    acc = torch.full((w.B,), -9, dtype=torch.int32, device="cuda")
+    ersd.ersd_gsd_verify(inp["target"].cuda(), inp["draft"].cuda(), tok, inp["seeds"].cuda(), inp["T"], out, acc)
+    torch.cuda.synchronize()
+    ref = oracle.gsd_verify(wl.as_numpy_logits(inp["target"]), wl.as_numpy_logits(inp["draft"]), tok.cpu().numpy(),
+                            wl.seeds_as_u64(inp["seeds"]), T=inp["T"])
+    ok = ~ambiguous(ref)
+    assert ok.sum() >= w.B - 1
+    assert (acc.cpu().numpy()[ok] == ref["accept_len"][ok]).all()
+    assert (out.cpu().numpy()[ok] == ref["tokens"][ok]).all()
+
+
+@pytest.mark.parametrize("off", [-2e-6, 2e-6])
+def test_ratio_tests_too_close_for_single_precision(ersd, off):
+    """Ratios 2e-6 away from their uniform number, far inside what single-precision sums can tell
+    (about 1e-5) and far outside what double precision cannot: every test takes the exact path."""
+    B, V = 64, 5000
+    g = torch.Generator().manual_seed(8)
+    drf = torch.randn(B, 1, V, generator=g, dtype=torch.float64)
+    x = torch.randint(0, V, (B, 1), generator=g)
+    seeds = wl.make_seeds(21, 0, B)
+    tok = x.to(torch.int32)
+    tgt = torch.randn(B, 2, V, generator=g).float()
+    first = oracle.gsd_verify(tgt.numpy(), drf.float().numpy(), tok.numpy(), wl.seeds_as_u64(seeds), T=1.0)
+    drf = drf.float()
+    d = drf[:, 0].double()
+    q = torch.softmax(d, -1).gather(1, x)[:, 0]
+    r = torch.from_numpy(first["unif"][:, 0]) * (1.0 + off)     # wanted ratio: the target law lifts or lowers token x alone
+    z = d.gather(1, x)[:, 0] + torch.log(r * (1 - q) / (1 - r * q))
+    t0 = d.clone()
+    t0.scatter_(1, x, z.unsqueeze(1))
+    tgt[:, 0] = t0.float()
+    out = torch.empty(B, 2, dtype=torch.int32, device="cuda")
+    acc = torch.empty(B, dtype=torch.int32, device="cuda")
+    ersd.ersd_gsd_verify(tgt.cuda(), drf.cuda(), tok.cuda(), seeds.cuda(), 1.0, out, acc)
+    torch.cuda.synchronize()
+    ref = oracle.gsd_verify(tgt.numpy(), drf.numpy(), tok.numpy(), wl.seeds_as_u64(seeds), T=1.0)
+    close = np.abs(ref["ratio"][:, 0] / ref["unif"][:, 0] - 1.0)
+    assert close.max() < 6e-6 and not ambiguous(ref).any()      # (float32 logits: the ratio is off by their rounding)
+    assert (acc.cpu().numpy() == ref["accept_len"]).all() and (out.cpu().numpy() == ref["tokens"]).all()
+
+
+def test_final_races_too_close_for_single_precision(ersd):
+    """Two tokens whose arrival times differ by 2e-5 relative: outside the near-tie window, inside the
+    intervals of the single-precision race."""
+    B, V = 64, 9000
+    g = torch.Generator().manual_seed(9)
+    tgt = torch.full((B, 1, V), float("-inf"))
+    a, b = torch.randint(0, 4000, (B,), generator=g), torch.randint(4000, V, (B,), generator=g)
+    n = torch.arange(B)
+    tgt[n, 0, a] = 0.0
+    tgt[n, 0, b] = 0.0
+    seeds = wl.make_seeds(22, 0, B)
+    none = np.zeros((B, 0), np.int32)
+    ref = oracle.gsd_verify(tgt.numpy(), np.zeros((B, 0, V), np.float32), none, wl.seeds_as_u64(seeds), T=1.0)
+    t, win = ref["last_times"], torch.from_numpy(ref["tokens"][:, 0].astype(np.int64))
+    other = torch.where(win == a, b, a)
+    tgt[n, 0, other] = torch.from_numpy(np.log(t[:, 1] / t[:, 0]) - 2e-5).float()    # the later one draws level
+    ref = oracle.gsd_verify(tgt.numpy(), np.zeros((B, 0, V), np.float32), none, wl.seeds_as_u64(seeds), T=1.0)
+    gap = ref["last_times"][:, 1] / ref["last_times"][:, 0] - 1.0
+    ok = gap > 1e-5
+    assert gap.max() < 4e-5 and ok.sum() > B // 2
+    out = torch.empty(B, 1, dtype=torch.int32, device="cuda")
+    acc = torch.empty(B, dtype=torch.int32, device="cuda")
+    ersd.ersd_gsd_verify(tgt.cuda(), None, None, seeds.cuda(), 1.0, out, acc)
+    torch.cuda.synchronize()
+    assert (acc == 0).all() and (out.cpu().numpy()[ok] == ref["tokens"][ok]).all()
