@@ -18,6 +18,7 @@
 #include <string.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "ersd.h"
 #include "ersd_math.cuh"
@@ -437,8 +438,8 @@ constexpr size_t kClusterSmemBytes = 200 * 1024;  // dynamic shared memory a blo
 
 // Tiles per block that fit (roles = rows raced together: 1, or 2 for a draft/target pair; cmax > 1:
 // the kernel for races of several arrivals, which keeps its lists behind the rows).
-static int cluster_max_tiles(int dt, int roles, int cmax) {
-  const size_t per_tile = dt == ERSD_BF16 ? b256::cluster_role_bytes<ERSD_BF16>(1) : b256::cluster_role_bytes<ERSD_F32>(1);
+static int cluster_max_tiles(int dt, int roles, int cmax, bool aligned) {
+  const size_t per_tile = dt == ERSD_BF16 ? b256::cluster_role_bytes<ERSD_BF16>(1, aligned) : b256::cluster_role_bytes<ERSD_F32>(1, aligned);
   const size_t lists = cmax > 1 ? b256::top_list_bytes(cmax, b256::kClusterMax) : 0;
   return (int)((kClusterSmemBytes - lists) / (per_tile * (size_t)roles));
 }
@@ -454,15 +455,21 @@ static int cluster_limit(int* out) {
   if (dev < 0 || dev >= 64) return ERSD_EUNSUPPORTED;
   std::lock_guard<std::mutex> lock(m);
   if (!limit[dev]) {
-    constexpr int kKernels = 8;
-    const void* kernels[kKernels] = {(const void*)b256::ersd_cluster_kernel<ERSD_BF16, 1>,
-                                     (const void*)b256::ersd_cluster_kernel<ERSD_F32, 1>,
-                                     (const void*)b256::ersd_cluster_kernel<ERSD_BF16, 2>,
-                                     (const void*)b256::ersd_cluster_kernel<ERSD_F32, 2>,
-                                     (const void*)b256::ersd_cluster_top_kernel<ERSD_BF16, 1>,
-                                     (const void*)b256::ersd_cluster_top_kernel<ERSD_F32, 1>,
-                                     (const void*)b256::ersd_cluster_top_kernel<ERSD_BF16, 2>,
-                                     (const void*)b256::ersd_cluster_top_kernel<ERSD_F32, 2>};
+    constexpr int kKernels = 16;
+    const void* kernels[kKernels];
+    int count = 0;
+    auto add = [&](auto dt, auto nr, auto al) {
+      kernels[count++] = (const void*)b256::ersd_cluster_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value>;
+      kernels[count++] = (const void*)b256::ersd_cluster_top_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value>;
+    };
+    auto both = [&](auto dt, auto nr) {
+      add(dt, nr, std::true_type());
+      add(dt, nr, std::false_type());
+    };
+    both(std::integral_constant<int, ERSD_BF16>(), std::integral_constant<int, 1>());
+    both(std::integral_constant<int, ERSD_BF16>(), std::integral_constant<int, 2>());
+    both(std::integral_constant<int, ERSD_F32>(), std::integral_constant<int, 1>());
+    both(std::integral_constant<int, ERSD_F32>(), std::integral_constant<int, 2>());
     int lim = 16;
     for (int q = 0; q < kKernels; ++q) {
       e = cudaFuncSetAttribute(kernels[q], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmemBytes);
@@ -502,13 +509,13 @@ static bool cluster_applies(const Params& p, int dt, int cmax) {
   const int roles = (p.mode == kVerify && p.draft) ? 2 : 1;
   const int64_t ntiles = ((int64_t)p.V + b256::kTile - 1) / b256::kTile;
   if (top && cmax > b256::kTopMaxC) return false;
-  if (ntiles > 8 * (int64_t)cluster_max_tiles(dt, roles, cmax)) return false;
+  if (ntiles > 8 * (int64_t)cluster_max_tiles(dt, roles, cmax, p.aligned_t && p.aligned_d)) return false;
   if (top) {
     if (p.given_tok || p.chain_outputs || p.extra) return false;
   } else if (p.mode == kVerify && p.rows > 32) {
     return false;
   }
-  return p.aligned_t && (roles == 1 || p.aligned_d) && p.rows <= 65535 && p.B <= 65535;
+  return p.rows <= 65535 && p.B <= 65535;
 }
 
 // Blocks per cluster.  Few positions: the smallest power of two that leaves a block about
@@ -521,7 +528,7 @@ static int cluster_size(const ersd_opts& o, const Params& p, int dt, int cmax, i
   if (ls != ERSD_OK) return ls;
   const int ntiles = (p.V + b256::kTile - 1) / b256::kTile;
   const int roles = (p.mode == kVerify && p.draft) ? 2 : 1;
-  const int max_tiles = cluster_max_tiles(dt, roles, cmax);
+  const int max_tiles = cluster_max_tiles(dt, roles, cmax, p.aligned_t && p.aligned_d);
   if (o.split_v) {  // the caller's choice: a power of two that the device takes and whose blocks can stage their share
     const int CL = (int)o.split_v;
     if (CL > lim || (CL & (CL - 1)) != 0 || (ntiles + CL - 1) / CL > max_tiles) return ERSD_EUNSUPPORTED;
@@ -556,7 +563,7 @@ static bool cluster_by_default(const ersd_opts& o, const Params& p, int dt, int 
   return blocks <= kClusterAutoBlocksSample;
 }
 
-template <int DT>
+template <int DT, bool AL>
 static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeDesc& tree, int cmax, cudaStream_t st) {
   Params p = p_in;
   p.top_cmax = cmax;
@@ -575,7 +582,7 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
     const int64_t rows_in_all = (int64_t)p.B * (p.rows + with_children);
     bool split = rows_in_all * CL <= kClusterSplitBlocks;
     if (!split && !o.split_v && CL >= 2 && rows_in_all * (CL / 2) <= kClusterSplitBlocks &&
-        (ntiles + CL / 2 - 1) / (CL / 2) <= cluster_max_tiles(DT, 1, cmax)) {
+        (ntiles + CL / 2 - 1) / (CL / 2) <= cluster_max_tiles(DT, 1, cmax, AL)) {
       CL /= 2;  // (a row to a cluster of half as many blocks)
       split = true;
     }
@@ -590,7 +597,7 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   memset(&cfg, 0, sizeof cfg);
   cfg.gridDim = dim3((unsigned)CL, (unsigned)jobs, (unsigned)p.B);
   cfg.blockDim = dim3(b256::kThreads, 1, 1);
-  cfg.dynamicSmemBytes = b256::cluster_role_bytes<DT>(G) * (size_t)roles + (cmax > 1 ? b256::top_list_bytes(cmax, CL) : 0);
+  cfg.dynamicSmemBytes = b256::cluster_role_bytes<DT>(G, AL) * (size_t)roles + (cmax > 1 ? b256::top_list_bytes(cmax, CL) : 0);
   cfg.stream = st;
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeClusterDimension;
@@ -604,18 +611,21 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
            p.B * jobs, CL, b256::kThreads, p.B * p.rows);
   cudaError_t e;
   if (cmax > 1) {
-    auto kernel = roles == 2 ? b256::ersd_cluster_top_kernel<DT, 2> : b256::ersd_cluster_top_kernel<DT, 1>;
+    auto kernel = roles == 2 ? b256::ersd_cluster_top_kernel<DT, 2, AL> : b256::ersd_cluster_top_kernel<DT, 1, AL>;
     e = cudaLaunchKernelEx(&cfg, kernel, p, tree);
   } else {
-    auto kernel = roles == 2 ? b256::ersd_cluster_kernel<DT, 2> : b256::ersd_cluster_kernel<DT, 1>;
+    auto kernel = roles == 2 ? b256::ersd_cluster_kernel<DT, 2, AL> : b256::ersd_cluster_kernel<DT, 1, AL>;
     e = cudaLaunchKernelEx(&cfg, kernel, p);
   }
   return e == cudaSuccess ? ERSD_OK : cuda_fail(e);
 }
 
 static int launch_cluster(const ersd_opts& o, const Params& p, const TreeDesc& tree, int dt, int cmax, cudaStream_t st) {
-  return dt == ERSD_BF16 ? launch_cluster_dt<ERSD_BF16>(o, p, tree, cmax, st)
-                         : launch_cluster_dt<ERSD_F32>(o, p, tree, cmax, st);
+  if (p.aligned_t && p.aligned_d)
+    return dt == ERSD_BF16 ? launch_cluster_dt<ERSD_BF16, true>(o, p, tree, cmax, st)
+                           : launch_cluster_dt<ERSD_F32, true>(o, p, tree, cmax, st);
+  return dt == ERSD_BF16 ? launch_cluster_dt<ERSD_BF16, false>(o, p, tree, cmax, st)
+                         : launch_cluster_dt<ERSD_F32, false>(o, p, tree, cmax, st);
 }
 
 static int check_common(const void* logits, int dt, const uint64_t* seeds, int B, int rows, int V,
@@ -683,7 +693,8 @@ static int verify_impl(const void* target, const void* draft, int dt, const Tree
   // kernel only: the cluster kernels keep no arrival beyond those asked for)
   if (o.kernel_path > 2) return ERSD_EINVAL;
   const bool cluster_ok = !p.extra && cluster_applies(p, dt, cmax);  // (a tree without branching is the chain 0 -> 1 -> ...)
-  if (o.kernel_path == 2 && !cluster_ok) return ERSD_EUNSUPPORTED;
+  // (asked for by name it is for rows on 16-byte boundaries, as documented)
+  if (o.kernel_path == 2 && !(cluster_ok && p.aligned_t && p.aligned_d)) return ERSD_EUNSUPPORTED;
   if (o.block_threads != 0 && o.block_threads != 128 && o.block_threads != 256) return ERSD_EINVAL;
   if (o.workspace) {
     if (o.workspace_bytes < workspace_bytes(B, rows)) return ERSD_EWORKSPACE;
@@ -824,7 +835,8 @@ int ersd_race_sample(const void* logits, ersd_dtype dt, const uint64_t* seeds, i
   if (o.kernel_path > 2) return ERSD_EINVAL;
   // (near-ties are counted by the streaming kernel only: the cluster kernels keep no arrival beyond those asked for)
   const bool cluster_ok = !extra && cluster_applies(p, dt, c);
-  if (o.kernel_path == 2 && !cluster_ok) return ERSD_EUNSUPPORTED;
+  // (asked for by name it is for rows on 16-byte boundaries, as documented)
+  if (o.kernel_path == 2 && !(cluster_ok && p.aligned_t)) return ERSD_EUNSUPPORTED;
   TreeDesc tree;
   memset(&tree, 0, sizeof tree);
   if (cluster_ok && (o.kernel_path == 2 || cluster_by_default(o, p, dt, c)))
