@@ -135,6 +135,9 @@ constexpr int kThreads = 128, kMinBlocks = 7;
 constexpr bool kMany = true;
 #include "ersd_kernel.inc"
 }  // namespace b128m
+namespace b128 {
+#include "ersd_cluster.inc"
+}  // namespace b128
 namespace b256 {
 #include "ersd_cluster.inc"
 #include "ersd_cluster_top.inc"
@@ -425,11 +428,24 @@ static int launch(const Params& p, const TreeDesc& tree, int dt, int cmax, cudaS
 // ---------------------------------------------------------------------------------------------
 // Latency path of calls of few rows: one cluster of thread blocks per position (ersd_cluster.inc).
 // ---------------------------------------------------------------------------------------------
-// Default choice: the cluster kernel is taken while its blocks number up to 1280 (sampling: 160
-// rows of 128256 logits) or, in verification (two rows per position), while the positions would
-// make up to 704 blocks in clusters of full size (44 positions of 128256 logits); beyond that the
-// streaming kernel's throughput wins (measured at V = 128256 and 32000).
-constexpr int64_t kClusterAutoBlocksSample = 1280, kClusterAutoBlocksVerify = 704;
+// Default choice for races of one arrival, by the logits of the call (positions x V).  Short rows
+// always take the cluster kernel, longer ones up to a number of logits from which the streaming
+// kernel's throughput wins (measured with rows of eleven lengths from 1024 to 128256.  Verification,
+// bf16: at 16384 logits 800 positions take 34.3 us here and 37.5 streamed, 1200 48.6 and 46.8; at
+// 32000 200 positions 24.8 and 25.9, 300 30.0 and 29.4; at 128256 50 24.9 and 25.7, 100 39.4 and 34.5.
+// Sampling, one row per position: at 32000 1200 rows 52.5 and 55.2 us, at 128256 150 rows 30.0 and
+// 36.1, 200 39.6 and 38.6.  32-bit logits take twice the room: verification at 4096 logits 3200
+// positions 53.8 and 63.4 us, at 8192 400 23.7 and 23.2, at 32000 100 27.6 and 24.9; sampling at
+// 32000 100 rows 14.6 and 18.7, 400 38.2 and 26.9).
+struct ClusterLimit {
+  int row;         // rows of up to this many logits ...
+  int64_t logits;  // ... take the cluster kernel while the call has no more logits than this
+};
+constexpr ClusterLimit kClusterLimits[2][2][3] = {
+    // ERSD_F32: one row per position, draft and target row
+    {{{8192, INT64_MAX}, {16384, 18 << 20}, {INT32_MAX, 5 << 20}}, {{4096, INT64_MAX}, {8192, 8 << 20}, {INT32_MAX, 2 << 20}}},
+    // ERSD_BF16
+    {{{16384, INT64_MAX}, {32768, 36 << 20}, {INT32_MAX, 20 << 20}}, {{8192, INT64_MAX}, {16384, 16 << 20}, {INT32_MAX, 8 << 20}}}};
 // The same for races of several arrivals (ersd_cluster_top.inc; three blocks per SM).
 constexpr int64_t kClusterAutoBlocksTop = 600;
 // ... and the number of blocks up to which a tree's rows get a cluster each (one block per SM and a half)
@@ -455,12 +471,13 @@ static int cluster_limit(int* out) {
   if (dev < 0 || dev >= 64) return ERSD_EUNSUPPORTED;
   std::lock_guard<std::mutex> lock(m);
   if (!limit[dev]) {
-    constexpr int kKernels = 16;
-    const void* kernels[kKernels];
-    int count = 0;
+    constexpr int kKernels = 16, kSmall = 8;  // (the last kSmall: 128-thread blocks, never in clusters)
+    const void* kernels[kKernels + kSmall];
+    int count = 0, small = kKernels;
     auto add = [&](auto dt, auto nr, auto al) {
       kernels[count++] = (const void*)b256::ersd_cluster_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value>;
       kernels[count++] = (const void*)b256::ersd_cluster_top_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value>;
+      kernels[small++] = (const void*)b128::ersd_cluster_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value>;
     };
     auto both = [&](auto dt, auto nr) {
       add(dt, nr, std::true_type());
@@ -471,7 +488,7 @@ static int cluster_limit(int* out) {
     both(std::integral_constant<int, ERSD_F32>(), std::integral_constant<int, 1>());
     both(std::integral_constant<int, ERSD_F32>(), std::integral_constant<int, 2>());
     int lim = 16;
-    for (int q = 0; q < kKernels; ++q) {
+    for (int q = 0; q < kKernels + kSmall; ++q) {
       e = cudaFuncSetAttribute(kernels[q], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmemBytes);
       if (e != cudaSuccess) return cuda_fail(e);
     }
@@ -552,15 +569,9 @@ static bool cluster_by_default(const ersd_opts& o, const Params& p, int dt, int 
   if (cluster_size(o, p, dt, cmax, &CL) != ERSD_OK) return false;
   const int64_t blocks = (int64_t)p.B * p.rows * CL;
   if (cmax > 1) return blocks <= kClusterAutoBlocksTop;
-  if (p.mode == kVerify) {
-    // counted in clusters of the size a lone position would get (16 blocks at V = 128256, 4 at
-    // 32000), whatever size this call's clusters have: 44 and 176 positions at those two sizes
-    const int ntiles = (p.V + b256::kTile - 1) / b256::kTile;
-    int full = 1;
-    while (full < b256::kClusterMax && full * b256::kClusterGroups < ntiles) full *= 2;
-    return (int64_t)p.B * p.rows * full <= kClusterAutoBlocksVerify;
-  }
-  return blocks <= kClusterAutoBlocksSample;
+  const ClusterLimit* limit = kClusterLimits[dt == ERSD_BF16][p.mode == kVerify && p.draft];
+  while (p.V > limit->row) ++limit;
+  return (int64_t)p.V * p.B * p.rows <= limit->logits;
 }
 
 template <int DT, bool AL>
@@ -592,12 +603,21 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
       roles = 1;
     }
   }
-  const int G = (ntiles + CL - 1) / CL;  // tiles per block; they fit, see cluster_applies
+  // Positions of one block each: blocks of 128 threads, twice as many to an SM, once there are more
+  // positions than 256-thread blocks would be resident (3200 rows of 2048 bf16 logits: sampling 19.6
+  // instead of 25.0 us, verification 26.8 instead of 37.0; at 400 rows equal; blocks of 64 threads
+  // 19.6 and 29.9), and for rows that 128 threads take in one turn (400 positions of 1024 logits: 8.4
+  // instead of 10.4 us); not where the staged rows would leave fewer than five such blocks to an SM.
+  const int G128 = (p.V + b128::kTile - 1) / b128::kTile;
+  const bool small = cmax == 1 && CL == 1 && b128::cluster_role_bytes<DT>(G128, AL) * (size_t)roles <= 41 * 1024 &&
+                     ((int64_t)p.B * p.rows > 4 * sm_count() || G128 == 1);
+  const int threads = small ? b128::kThreads : b256::kThreads;
+  const int G = small ? G128 : (ntiles + CL - 1) / CL;  // tiles per block; they fit, see cluster_applies
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
   cfg.gridDim = dim3((unsigned)CL, (unsigned)jobs, (unsigned)p.B);
-  cfg.blockDim = dim3(b256::kThreads, 1, 1);
-  cfg.dynamicSmemBytes = b256::cluster_role_bytes<DT>(G, AL) * (size_t)roles + (cmax > 1 ? b256::top_list_bytes(cmax, CL) : 0);
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = (small ? b128::cluster_role_bytes<DT>(G, AL) : b256::cluster_role_bytes<DT>(G, AL)) * (size_t)roles + (cmax > 1 ? b256::top_list_bytes(cmax, CL) : 0);
   cfg.stream = st;
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeClusterDimension;
@@ -608,13 +628,14 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   cfg.numAttrs = 1;
   snprintf(g_last_launch, sizeof g_last_launch, "%s<%s, %d row(s) per cluster>: %d clusters of %d x %d threads, %d positions",
            cmax > 1 ? "ersd_cluster_top_kernel" : "ersd_cluster_kernel", DT == ERSD_BF16 ? "bf16" : "f32", roles,
-           p.B * jobs, CL, b256::kThreads, p.B * p.rows);
+           p.B * jobs, CL, threads, p.B * p.rows);
   cudaError_t e;
   if (cmax > 1) {
     auto kernel = roles == 2 ? b256::ersd_cluster_top_kernel<DT, 2, AL> : b256::ersd_cluster_top_kernel<DT, 1, AL>;
     e = cudaLaunchKernelEx(&cfg, kernel, p, tree);
   } else {
     auto kernel = roles == 2 ? b256::ersd_cluster_kernel<DT, 2, AL> : b256::ersd_cluster_kernel<DT, 1, AL>;
+    if (small) kernel = roles == 2 ? b128::ersd_cluster_kernel<DT, 2, AL> : b128::ersd_cluster_kernel<DT, 1, AL>;
     e = cudaLaunchKernelEx(&cfg, kernel, p);
   }
   return e == cudaSuccess ? ERSD_OK : cuda_fail(e);

@@ -71,3 +71,20 @@ def test_few_rows_of_several_arrivals(ersd, V, dtype):
     torch.cuda.synchronize()
     assert "ersd_cluster_top_kernel" in ersd.ersd_last_launch()
     check_sample(logits, seeds, 0.9, tok, key, c=c)
+
+
+@pytest.mark.parametrize("V", [5, 1024, 1030, 3001])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_many_short_rows_take_small_blocks(ersd, V, dtype):
+    """More positions than 256-thread blocks are resident: one block of 128 threads per position."""
+    inp = inputs(150, 4, V, dtype)
+    out = run(ersd, inp)
+    assert "x 128 threads" in ersd.ersd_last_launch()
+    check_verify(inp, out)
+    logits, seeds = inp["target"], inp["seeds"]
+    tok = torch.full((150, 5, 1), -7, dtype=torch.int32, device="cuda")
+    key = torch.full((150, 5, 1), -7.0, dtype=torch.float32, device="cuda")
+    ersd.ersd_race_sample(logits.cuda(), seeds.cuda(), 0.8, tok, ersd.make_opts(out_key=key))
+    torch.cuda.synchronize()
+    assert "x 128 threads" in ersd.ersd_last_launch()
+    check_sample(logits, seeds, 0.8, tok, key)
