@@ -1,9 +1,11 @@
-"""Thin ctypes binding of libersd.so: argument marshalling only.
+"""Thin binding of libersd.so: argument marshalling only.
 
 The functions carry the names of the C entry points in ``include/ersd.h`` and
 take torch CUDA tensors (used for device memory and the current stream only).
-Every step of the computation runs in the library's kernels.  Loading fails
-loudly when the library has not been built: there is no CPU path.
+Every step of the computation runs in the library's kernels.  The calls of a
+decoding loop go through the extension module ``_ersd_call`` (checks, addresses,
+current stream and call in one step of native code), the others through ctypes.
+Loading fails loudly when either has not been built: there is no CPU path.
 """
 from __future__ import annotations
 
@@ -94,6 +96,26 @@ def lib():
     return _lib
 
 
+_native = None
+
+
+def native():
+    """The extension module that makes the calls, set to the loaded library's functions."""
+    global _native
+    if _native is None:
+        L = lib()
+        try:
+            from . import _ersd_call
+        except ImportError as e:
+            raise RuntimeError("_ersd_call.so not found next to %s: run `python -m paper_2504_15475_b200.build` (%s)"
+                               % (__file__, e)) from None
+        _ersd_call.use(*[C.cast(f, C.c_void_p).value for f in (
+            L.ersd_race_sample, L.ersd_verify, L.ersd_verify_noalloc, L.ersd_verify_tokens, L.ersd_verify_tree,
+            L.ersd_gsd_verify, L.ersd_gsd_verify_tree)])
+        _native = _ersd_call
+    return _native
+
+
 def _dtype_code(t: torch.Tensor) -> int:
     if t.dtype == torch.float32:
         return ERSD_F32
@@ -124,16 +146,6 @@ def _dev(t: torch.Tensor, dtype, name: str):
     if not t.is_contiguous():
         raise ValueError("%s must be contiguous" % name)
     return t
-
-
-def _sizes(logits: torch.Tensor, V: Optional[int]):
-    """(B, rows, V) of a logits tensor [B, rows, ld]; V defaults to ld (rows without padding)."""
-    B, rows, ld = logits.shape
-    if V is None:
-        return B, rows, ld
-    if not 1 <= int(V) <= ld:
-        raise ValueError("V must be between 1 and the row length of the tensor")
-    return B, rows, int(V)
 
 
 def make_opts(*, top_c: int = 0, split_v: int = 0, block_threads: int = 0, ld_target: int = 0, ld_draft: int = 0,
@@ -221,13 +233,9 @@ def ersd_race_sample(logits: torch.Tensor, seeds: torch.Tensor, T: float, out_to
                      opts: Optional[ErsdOpts] = None, stream=None, V: Optional[int] = None) -> None:
     """logits [B, R, V] (f32/bf16), seeds int64 [B] (the uint64 bit patterns), out_tok int32 [B, R, c].
     Padded rows: pass the tensor [B, R, ld], the vocabulary size as ``V`` and opts.ld_target = ld."""
-    _dev(logits, None, "logits")
-    _dev(seeds, torch.int64, "seeds")
-    _dev(out_tok, torch.int32, "out_tok")
-    B, R, V = _sizes(logits, V)
-    _check(lib().ersd_race_sample(_ptr(logits), _dtype_code(logits), _ptr(seeds), B, R, V, float(T),
-                                  _ptr(out_tok), C.byref(opts) if opts is not None else None,
-                                  _stream(stream)), "ersd_race_sample")
+    status = (_native or native()).race_sample(logits, seeds, T, out_tok, opts, stream, V)
+    if status:
+        raise ErsdError(status, "ersd_race_sample")
 
 
 def ersd_verify(target_logits: torch.Tensor, draft_logits: Optional[torch.Tensor], seeds: torch.Tensor,
@@ -235,17 +243,10 @@ def ersd_verify(target_logits: torch.Tensor, draft_logits: Optional[torch.Tensor
                 opts: Optional[ErsdOpts] = None, stream=None, V: Optional[int] = None) -> None:
     """target [B, k+1, V], draft [B, k, V], out_tokens int32 [B, k+1], out_accept_len int32 [B].
     Padded rows: tensors [B, rows, ld], the vocabulary size as ``V``, opts.ld_target / ld_draft = ld."""
-    _dev(target_logits, None, "target_logits")
-    B, rows, V = _sizes(target_logits, V)
-    if draft_logits is not None:
-        _dev(draft_logits, target_logits.dtype, "draft_logits")
-    _dev(seeds, torch.int64, "seeds")
-    _dev(out_tokens, torch.int32, "out_tokens")
-    _dev(out_accept_len, torch.int32, "out_accept_len")
-    _check(lib().ersd_verify(_ptr(target_logits), _ptr(draft_logits), _dtype_code(target_logits),
-                             _ptr(seeds), B, rows - 1, V, float(T), _ptr(out_tokens),
-                             _ptr(out_accept_len), C.byref(opts) if opts is not None else None,
-                             _stream(stream)), "ersd_verify")
+    status = (_native or native()).verify(target_logits, draft_logits, seeds, T, out_tokens, out_accept_len, opts,
+                                          stream, V)
+    if status:
+        raise ErsdError(status, "ersd_verify")
 
 
 def ersd_verify_tokens(target_logits: torch.Tensor, draft_tokens: Optional[torch.Tensor], seeds: torch.Tensor,
@@ -253,17 +254,10 @@ def ersd_verify_tokens(target_logits: torch.Tensor, draft_tokens: Optional[torch
                        opts: Optional[ErsdOpts] = None, stream=None, V: Optional[int] = None) -> None:
     """target [B, k+1, V], draft_tokens int32 [B, k] (drafted earlier with the same races),
     out_tokens int32 [B, k+1], out_accept_len int32 [B]."""
-    _dev(target_logits, None, "target_logits")
-    B, rows, V = _sizes(target_logits, V)
-    if draft_tokens is not None:
-        _dev(draft_tokens, torch.int32, "draft_tokens")
-    _dev(seeds, torch.int64, "seeds")
-    _dev(out_tokens, torch.int32, "out_tokens")
-    _dev(out_accept_len, torch.int32, "out_accept_len")
-    _check(lib().ersd_verify_tokens(_ptr(target_logits), _ptr(draft_tokens), _dtype_code(target_logits),
-                                    _ptr(seeds), B, rows - 1, V, float(T), _ptr(out_tokens),
-                                    _ptr(out_accept_len), C.byref(opts) if opts is not None else None,
-                                    _stream(stream)), "ersd_verify_tokens")
+    status = (_native or native()).verify_tokens(target_logits, draft_tokens, seeds, T, out_tokens, out_accept_len, opts,
+                                                 stream, V)
+    if status:
+        raise ErsdError(status, "ersd_verify_tokens")
 
 
 def ersd_gsd_verify(target_logits: torch.Tensor, draft_logits: Optional[torch.Tensor],
@@ -272,19 +266,10 @@ def ersd_gsd_verify(target_logits: torch.Tensor, draft_logits: Optional[torch.Te
                     V: Optional[int] = None) -> None:
     """Greedy speculative decoding (Algorithm 1 position by position) on the same logits.
     target [B, k+1, V], draft [B, k, V], draft_tokens int32 [B, k]; out_tokens int32 [B, k+1]."""
-    _dev(target_logits, None, "target_logits")
-    B, rows, V = _sizes(target_logits, V)
-    if draft_logits is not None:
-        _dev(draft_logits, target_logits.dtype, "draft_logits")
-    if draft_tokens is not None:
-        _dev(draft_tokens, torch.int32, "draft_tokens")
-    _dev(seeds, torch.int64, "seeds")
-    _dev(out_tokens, torch.int32, "out_tokens")
-    _dev(out_accept_len, torch.int32, "out_accept_len")
-    _check(lib().ersd_gsd_verify(_ptr(target_logits), _ptr(draft_logits), _ptr(draft_tokens),
-                                 _dtype_code(target_logits), _ptr(seeds), B, rows - 1, V, float(T),
-                                 _ptr(out_tokens), _ptr(out_accept_len),
-                                 C.byref(opts) if opts is not None else None, _stream(stream)), "ersd_gsd_verify")
+    status = (_native or native()).gsd_verify(target_logits, draft_logits, draft_tokens, seeds, T, out_tokens, out_accept_len,
+                                              opts, stream, V)
+    if status:
+        raise ErsdError(status, "ersd_gsd_verify")
 
 
 def ersd_gsd_verify_tree(target_logits: torch.Tensor, draft_logits: Optional[torch.Tensor],
@@ -293,21 +278,10 @@ def ersd_gsd_verify_tree(target_logits: torch.Tensor, draft_logits: Optional[tor
                          opts: Optional[ErsdOpts] = None, stream=None, V: Optional[int] = None) -> None:
     """Tree GSD (Algorithm 4).  target, draft [B, N+1, V]; draft_tokens int32 [B, N+1] (entry 0
     unused); parent: host list [N+1]; out_tokens int32 [B, D+1]."""
-    _dev(target_logits, None, "target_logits")
-    B, rows, V = _sizes(target_logits, V)
-    if draft_logits is not None:
-        _dev(draft_logits, target_logits.dtype, "draft_logits")
-    if draft_tokens is not None:
-        _dev(draft_tokens, torch.int32, "draft_tokens")
-    _dev(seeds, torch.int64, "seeds")
-    _dev(out_tokens, torch.int32, "out_tokens")
-    _dev(out_accept_len, torch.int32, "out_accept_len")
-    arr = (C.c_int32 * len(parent))(*[int(x) for x in parent])
-    _check(lib().ersd_gsd_verify_tree(_ptr(target_logits), _ptr(draft_logits), _ptr(draft_tokens),
-                                      _dtype_code(target_logits), arr, _ptr(seeds), B, rows - 1, V, float(T),
-                                      _ptr(out_tokens), _ptr(out_accept_len),
-                                      C.byref(opts) if opts is not None else None, _stream(stream)),
-           "ersd_gsd_verify_tree")
+    status = (_native or native()).gsd_verify_tree(target_logits, draft_logits, draft_tokens, parent, seeds, T, out_tokens,
+                                                   out_accept_len, opts, stream, V)
+    if status:
+        raise ErsdError(status, "ersd_gsd_verify_tree")
 
 
 def ersd_verify_noalloc(target_logits: torch.Tensor, draft_logits: Optional[torch.Tensor],
@@ -317,17 +291,10 @@ def ersd_verify_noalloc(target_logits: torch.Tensor, draft_logits: Optional[torc
     """ersd_verify for callers that cannot allocate device memory: same arguments and results,
     scratch built into the library, B * (k + 1) <= ERSD_NOALLOC_MAX_ROWS.  Calls on one device
     share that scratch, so they must not overlap on the GPU."""
-    _dev(target_logits, None, "target_logits")
-    B, rows, V = _sizes(target_logits, V)
-    if draft_logits is not None:
-        _dev(draft_logits, target_logits.dtype, "draft_logits")
-    _dev(seeds, torch.int64, "seeds")
-    _dev(out_tokens, torch.int32, "out_tokens")
-    _dev(out_accept_len, torch.int32, "out_accept_len")
-    _check(lib().ersd_verify_noalloc(_ptr(target_logits), _ptr(draft_logits), _dtype_code(target_logits),
-                                     _ptr(seeds), B, rows - 1, V, float(T), _ptr(out_tokens),
-                                     _ptr(out_accept_len), C.byref(opts) if opts is not None else None,
-                                     _stream(stream)), "ersd_verify_noalloc")
+    status = (_native or native()).verify_noalloc(target_logits, draft_logits, seeds, T, out_tokens, out_accept_len, opts,
+                                                  stream, V)
+    if status:
+        raise ErsdError(status, "ersd_verify_noalloc")
 
 
 def ersd_verify_tree(target_logits: torch.Tensor, draft_logits: Optional[torch.Tensor],
@@ -335,18 +302,10 @@ def ersd_verify_tree(target_logits: torch.Tensor, draft_logits: Optional[torch.T
                      out_accept_len: torch.Tensor, opts: Optional[ErsdOpts] = None, stream=None,
                      V: Optional[int] = None) -> None:
     """target, draft [B, N+1, V]; parent: host list [N+1]; out_tokens int32 [B, D+1]."""
-    _dev(target_logits, None, "target_logits")
-    B, nodes, V = _sizes(target_logits, V)
-    if draft_logits is not None:
-        _dev(draft_logits, target_logits.dtype, "draft_logits")
-    _dev(seeds, torch.int64, "seeds")
-    _dev(out_tokens, torch.int32, "out_tokens")
-    _dev(out_accept_len, torch.int32, "out_accept_len")
-    arr = (C.c_int32 * len(parent))(*[int(p) for p in parent])
-    _check(lib().ersd_verify_tree(_ptr(target_logits), _ptr(draft_logits), _dtype_code(target_logits),
-                                  arr, _ptr(seeds), B, nodes - 1, V, float(T), _ptr(out_tokens),
-                                  _ptr(out_accept_len), C.byref(opts) if opts is not None else None,
-                                  _stream(stream)), "ersd_verify_tree")
+    status = (_native or native()).verify_tree(target_logits, draft_logits, parent, seeds, T, out_tokens, out_accept_len, opts,
+                                               stream, V)
+    if status:
+        raise ErsdError(status, "ersd_verify_tree")
 
 
 def ersd_row_keys(row: torch.Tensor, T: float, seed: int, seq_id: int, position: int, mode: int,
