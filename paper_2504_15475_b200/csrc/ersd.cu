@@ -71,6 +71,15 @@ __device__ __forceinline__ uint4 bytes_from(const uint4& lo, const uint4& hi, un
                     __funnelshift_r(w[2], w[3], bits), __funnelshift_r(w[3], w[4], bits));
 }
 
+// Programmatic dependent launch: a kernel launched with the attribute starts while the kernel before
+// it on the stream still runs; everything it reads or writes in global memory comes after this wait,
+// which ends when that kernel has completed and its stores are visible.  Once past it the kernel lets
+// the next one start likewise, so that at most one launch waits on the device.
+__device__ __forceinline__ void wait_for_previous_kernel() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 enum Mode { kSample = 0, kVerify = 1 };
 
 struct Params {
@@ -176,6 +185,29 @@ static int cuda_fail(cudaError_t e) {
   g_last_cuda_error = (int)e;
   return ERSD_ECUDA;
 }
+
+// A launch that may start while the kernel before it on the stream still runs (see
+// wait_for_previous_kernel), in clusters of CL blocks.
+struct Launch {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at[2];
+  Launch(dim3 grid, unsigned threads, size_t smem, cudaStream_t st, unsigned CL = 1) {
+    memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = CL;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = CL > 1 ? 2 : 1;
+  }
+  Launch(const Launch&) = delete;
+};
 
 struct OwnedWorkspace {
   void* ptr = nullptr;
@@ -398,30 +430,18 @@ static int launch(const Params& p, const TreeDesc& tree, int dt, int cmax, cudaS
   if (pst != ERSD_OK) return pst;
   snprintf(g_last_launch, sizeof g_last_launch, "ersd_race_kernel<%s>%s: %d threads x (%d, %d, %d) blocks, %d chunk(s) per row",
            dt == ERSD_BF16 ? "bf16" : "f32", many ? " (pooled thresholds)" : "", p.threads, p.B, p.rows, p.S, p.S);
-  if (many) {
-    if (p.threads == 128) {
-      if (dt == ERSD_BF16)
-        b128m::ersd_race_kernel<ERSD_BF16><<<grid, 128, sizeof(b128m::Shared<ERSD_BF16>), st>>>(p, tree);
-      else
-        b128m::ersd_race_kernel<ERSD_F32><<<grid, 128, sizeof(b128m::Shared<ERSD_F32>), st>>>(p, tree);
-    } else {
-      if (dt == ERSD_BF16)
-        b256m::ersd_race_kernel<ERSD_BF16><<<grid, 256, sizeof(b256m::Shared<ERSD_BF16>), st>>>(p, tree);
-      else
-        b256m::ersd_race_kernel<ERSD_F32><<<grid, 256, sizeof(b256m::Shared<ERSD_F32>), st>>>(p, tree);
-    }
-  } else if (p.threads == 128) {
-    if (dt == ERSD_BF16)
-      b128::ersd_race_kernel<ERSD_BF16><<<grid, 128, sizeof(b128::Shared<ERSD_BF16>), st>>>(p, tree);
-    else
-      b128::ersd_race_kernel<ERSD_F32><<<grid, 128, sizeof(b128::Shared<ERSD_F32>), st>>>(p, tree);
-  } else {
-    if (dt == ERSD_BF16)
-      b256::ersd_race_kernel<ERSD_BF16><<<grid, 256, sizeof(b256::Shared<ERSD_BF16>), st>>>(p, tree);
-    else
-      b256::ersd_race_kernel<ERSD_F32><<<grid, 256, sizeof(b256::Shared<ERSD_F32>), st>>>(p, tree);
-  }
-  const cudaError_t e = cudaGetLastError();
+  const bool small = p.threads == 128, bf16 = dt == ERSD_BF16;
+  void (*kernel)(Params, TreeDesc) =
+      many ? (small ? (bf16 ? b128m::ersd_race_kernel<ERSD_BF16> : b128m::ersd_race_kernel<ERSD_F32>)
+                    : (bf16 ? b256m::ersd_race_kernel<ERSD_BF16> : b256m::ersd_race_kernel<ERSD_F32>))
+           : (small ? (bf16 ? b128::ersd_race_kernel<ERSD_BF16> : b128::ersd_race_kernel<ERSD_F32>)
+                    : (bf16 ? b256::ersd_race_kernel<ERSD_BF16> : b256::ersd_race_kernel<ERSD_F32>));
+  const size_t smem = many ? (small ? (bf16 ? sizeof(b128m::Shared<ERSD_BF16>) : sizeof(b128m::Shared<ERSD_F32>))
+                                    : (bf16 ? sizeof(b256m::Shared<ERSD_BF16>) : sizeof(b256m::Shared<ERSD_F32>)))
+                           : (small ? (bf16 ? sizeof(b128::Shared<ERSD_BF16>) : sizeof(b128::Shared<ERSD_F32>))
+                                    : (bf16 ? sizeof(b256::Shared<ERSD_BF16>) : sizeof(b256::Shared<ERSD_F32>)));
+  Launch l(grid, (unsigned)p.threads, smem, st);
+  const cudaError_t e = cudaLaunchKernelEx(&l.cfg, kernel, p, tree);
   return e == cudaSuccess ? ERSD_OK : cuda_fail(e);
 }
 
@@ -613,30 +633,20 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
                      ((int64_t)p.B * p.rows > 4 * sm_count() || G128 == 1);
   const int threads = small ? b128::kThreads : b256::kThreads;
   const int G = small ? G128 : (ntiles + CL - 1) / CL;  // tiles per block; they fit, see cluster_applies
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof cfg);
-  cfg.gridDim = dim3((unsigned)CL, (unsigned)jobs, (unsigned)p.B);
-  cfg.blockDim = dim3(threads, 1, 1);
-  cfg.dynamicSmemBytes = (small ? b128::cluster_role_bytes<DT>(G, AL) : b256::cluster_role_bytes<DT>(G, AL)) * (size_t)roles + (cmax > 1 ? b256::top_list_bytes(cmax, CL) : 0);
-  cfg.stream = st;
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = (unsigned)CL;
-  at.val.clusterDim.y = 1;
-  at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  const size_t smem = (small ? b128::cluster_role_bytes<DT>(G, AL) : b256::cluster_role_bytes<DT>(G, AL)) * (size_t)roles +
+                      (cmax > 1 ? b256::top_list_bytes(cmax, CL) : 0);
+  Launch l(dim3((unsigned)CL, (unsigned)jobs, (unsigned)p.B), (unsigned)threads, smem, st, (unsigned)CL);
   snprintf(g_last_launch, sizeof g_last_launch, "%s<%s, %d row(s) per cluster>: %d clusters of %d x %d threads, %d positions",
            cmax > 1 ? "ersd_cluster_top_kernel" : "ersd_cluster_kernel", DT == ERSD_BF16 ? "bf16" : "f32", roles,
            p.B * jobs, CL, threads, p.B * p.rows);
   cudaError_t e;
   if (cmax > 1) {
     auto kernel = roles == 2 ? b256::ersd_cluster_top_kernel<DT, 2, AL> : b256::ersd_cluster_top_kernel<DT, 1, AL>;
-    e = cudaLaunchKernelEx(&cfg, kernel, p, tree);
+    e = cudaLaunchKernelEx(&l.cfg, kernel, p, tree);
   } else {
     auto kernel = roles == 2 ? b256::ersd_cluster_kernel<DT, 2, AL> : b256::ersd_cluster_kernel<DT, 1, AL>;
     if (small) kernel = roles == 2 ? b128::ersd_cluster_kernel<DT, 2, AL> : b128::ersd_cluster_kernel<DT, 1, AL>;
-    e = cudaLaunchKernelEx(&cfg, kernel, p);
+    e = cudaLaunchKernelEx(&l.cfg, kernel, p);
   }
   return e == cudaSuccess ? ERSD_OK : cuda_fail(e);
 }
@@ -1006,14 +1016,10 @@ int ersd_gsd_verify(const void* target_logits, const void* draft_logits, const i
   const int per_block = kGsdStatsThreads / 32;  // slices of a block of the sums
   const dim3 sums_grid((unsigned)(2 * k + 1), (unsigned)B, (unsigned)((g.S1 + per_block - 1) / per_block));
   const dim3 race_grid((unsigned)g.S, (unsigned)B);
-  if (dt == ERSD_BF16) {
-    gsd_stats_kernel<ERSD_BF16><<<sums_grid, kGsdStatsThreads, 0, stream>>>(g);
-    gsd_race_kernel<ERSD_BF16><<<race_grid, kGsdThreads, 0, stream>>>(g);
-  } else {
-    gsd_stats_kernel<ERSD_F32><<<sums_grid, kGsdStatsThreads, 0, stream>>>(g);
-    gsd_race_kernel<ERSD_F32><<<race_grid, kGsdThreads, 0, stream>>>(g);
-  }
-  const cudaError_t e = cudaGetLastError();
+  const bool bf16 = dt == ERSD_BF16;
+  Launch sums(sums_grid, kGsdStatsThreads, 0, stream), race(race_grid, kGsdThreads, 0, stream);
+  cudaError_t e = cudaLaunchKernelEx(&sums.cfg, bf16 ? gsd_stats_kernel<ERSD_BF16> : gsd_stats_kernel<ERSD_F32>, g);
+  if (e == cudaSuccess) e = cudaLaunchKernelEx(&race.cfg, bf16 ? gsd_race_kernel<ERSD_BF16> : gsd_race_kernel<ERSD_F32>, g);
   return e == cudaSuccess ? ERSD_OK : cuda_fail(e);
 }
 
