@@ -381,6 +381,23 @@ static int build_tree(const int32_t* parent, int N, TreeDesc* t, int* depth_out,
   return ERSD_OK;
 }
 
+// The build of the race kernel for a call, and its dynamic shared memory.
+struct RaceKernel {
+  void (*kernel)(Params, TreeDesc);
+  size_t smem;
+};
+template <int DT, bool AL>
+static RaceKernel race_kernel_of(bool many, int threads) {
+  if (many) return threads == 128 ? RaceKernel{b128m::ersd_race_kernel<DT, AL>, sizeof(b128m::Shared<DT>)}
+                                  : RaceKernel{b256m::ersd_race_kernel<DT, AL>, sizeof(b256m::Shared<DT>)};
+  return threads == 128 ? RaceKernel{b128::ersd_race_kernel<DT, AL>, sizeof(b128::Shared<DT>)}
+                        : RaceKernel{b256::ersd_race_kernel<DT, AL>, sizeof(b256::Shared<DT>)};
+}
+static RaceKernel race_kernel(bool bf16, bool aligned, bool many, int threads) {
+  if (bf16) return aligned ? race_kernel_of<ERSD_BF16, true>(many, threads) : race_kernel_of<ERSD_BF16, false>(many, threads);
+  return aligned ? race_kernel_of<ERSD_F32, true>(many, threads) : race_kernel_of<ERSD_F32, false>(many, threads);
+}
+
 // Four resident blocks per SM need about 180 KB of shared memory: ask for the largest carveout
 // (a hint to the driver; set once per device and kernel).
 static int prefer_shared_memory() {
@@ -393,20 +410,18 @@ static int prefer_shared_memory() {
   std::lock_guard<std::mutex> lock(m);
   if (!done[dev]) {
     e = cudaSuccess;
-    const void* kernels[8] = {(const void*)b256::ersd_race_kernel<ERSD_BF16>, (const void*)b256::ersd_race_kernel<ERSD_F32>,
-                              (const void*)b128::ersd_race_kernel<ERSD_BF16>, (const void*)b128::ersd_race_kernel<ERSD_F32>,
-                              (const void*)b256m::ersd_race_kernel<ERSD_BF16>, (const void*)b256m::ersd_race_kernel<ERSD_F32>,
-                              (const void*)b128m::ersd_race_kernel<ERSD_BF16>, (const void*)b128m::ersd_race_kernel<ERSD_F32>};
-    const int smem[8] = {(int)sizeof(b256::Shared<ERSD_BF16>), (int)sizeof(b256::Shared<ERSD_F32>),
-                         (int)sizeof(b128::Shared<ERSD_BF16>), (int)sizeof(b128::Shared<ERSD_F32>),
-                         (int)sizeof(b256m::Shared<ERSD_BF16>), (int)sizeof(b256m::Shared<ERSD_F32>),
-                         (int)sizeof(b128m::Shared<ERSD_BF16>), (int)sizeof(b128m::Shared<ERSD_F32>)};
-    for (int q = 0; q < 8 && e == cudaSuccess; ++q) {
-      e = cudaFuncSetAttribute(kernels[q], cudaFuncAttributePreferredSharedMemoryCarveout,
-                               cudaSharedmemCarveoutMaxShared);
+    auto prefer = [&](const void* kernel, size_t smem) {
       if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kernels[q], cudaFuncAttributeMaxDynamicSharedMemorySize, smem[q]);
-    }
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    };
+    for (int bf16 = 0; bf16 < 2; ++bf16)
+      for (int aligned = 0; aligned < 2; ++aligned)
+        for (int many = 0; many < 2; ++many)
+          for (int threads = 128; threads <= 256; threads += 128) {
+            const RaceKernel k = race_kernel(bf16 != 0, aligned != 0, many != 0, threads);
+            prefer((const void*)k.kernel, k.smem);
+          }
     if (e != cudaSuccess) return cuda_fail(e);
     done[dev] = true;
   }
@@ -430,18 +445,9 @@ static int launch(const Params& p, const TreeDesc& tree, int dt, int cmax, cudaS
   if (pst != ERSD_OK) return pst;
   snprintf(g_last_launch, sizeof g_last_launch, "ersd_race_kernel<%s>%s: %d threads x (%d, %d, %d) blocks, %d chunk(s) per row",
            dt == ERSD_BF16 ? "bf16" : "f32", many ? " (pooled thresholds)" : "", p.threads, p.B, p.rows, p.S, p.S);
-  const bool small = p.threads == 128, bf16 = dt == ERSD_BF16;
-  void (*kernel)(Params, TreeDesc) =
-      many ? (small ? (bf16 ? b128m::ersd_race_kernel<ERSD_BF16> : b128m::ersd_race_kernel<ERSD_F32>)
-                    : (bf16 ? b256m::ersd_race_kernel<ERSD_BF16> : b256m::ersd_race_kernel<ERSD_F32>))
-           : (small ? (bf16 ? b128::ersd_race_kernel<ERSD_BF16> : b128::ersd_race_kernel<ERSD_F32>)
-                    : (bf16 ? b256::ersd_race_kernel<ERSD_BF16> : b256::ersd_race_kernel<ERSD_F32>));
-  const size_t smem = many ? (small ? (bf16 ? sizeof(b128m::Shared<ERSD_BF16>) : sizeof(b128m::Shared<ERSD_F32>))
-                                    : (bf16 ? sizeof(b256m::Shared<ERSD_BF16>) : sizeof(b256m::Shared<ERSD_F32>)))
-                           : (small ? (bf16 ? sizeof(b128::Shared<ERSD_BF16>) : sizeof(b128::Shared<ERSD_F32>))
-                                    : (bf16 ? sizeof(b256::Shared<ERSD_BF16>) : sizeof(b256::Shared<ERSD_F32>)));
-  Launch l(grid, (unsigned)p.threads, smem, st);
-  const cudaError_t e = cudaLaunchKernelEx(&l.cfg, kernel, p, tree);
+  const RaceKernel k = race_kernel(dt == ERSD_BF16, p.aligned_t && p.aligned_d, many, p.threads);
+  Launch l(grid, (unsigned)p.threads, k.smem, st);
+  const cudaError_t e = cudaLaunchKernelEx(&l.cfg, k.kernel, p, tree);
   return e == cudaSuccess ? ERSD_OK : cuda_fail(e);
 }
 

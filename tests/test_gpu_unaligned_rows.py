@@ -88,3 +88,19 @@ def test_many_short_rows_take_small_blocks(ersd, V, dtype):
     torch.cuda.synchronize()
     assert "x 128 threads" in ersd.ersd_last_launch()
     check_sample(logits, seeds, 0.8, tok, key)
+
+
+@pytest.mark.parametrize("threads", [128, 256])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("V", [3, 1027, 2055, 4097, 8199, 16390, 40001])
+def test_streaming_kernel(ersd, V, dtype, threads):
+    """The ring over memory's 16-byte units: chunks of few tiles, two ragged tiles at a row's end, every shift."""
+    inp = inputs(4, 3, V, dtype)
+    for split in (0, 3):
+        out = run(ersd, inp, kernel_path=1, block_threads=threads, split_v=split)
+        assert "ersd_race_kernel" in ersd.ersd_last_launch()
+        check_verify(inp, out)
+    tree = inputs(2, len(wl.TREE_4x4) - 1, V, dtype, parent=wl.TREE_4x4)
+    out = run(ersd, tree, kernel_path=1, block_threads=threads)
+    assert "ersd_race_kernel" in ersd.ersd_last_launch()
+    check_verify(tree, out)
