@@ -73,12 +73,12 @@ __device__ __forceinline__ uint4 bytes_from(const uint4& lo, const uint4& hi, un
 
 // Programmatic dependent launch: a kernel launched with the attribute starts while the kernel before
 // it on the stream still runs; everything it reads or writes in global memory comes after this wait,
-// which ends when that kernel has completed and its stores are visible.  Once past it the kernel lets
-// the next one start likewise, so that at most one launch waits on the device.
-__device__ __forceinline__ void wait_for_previous_kernel() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+// which ends when that kernel has completed and its stores are visible.
+__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next kernel start once every block of this one has come here (without it: when this one has
+// ended, which still spares it most of a launch's latency).  Called past the wait, so that at most one
+// launch waits on the device.
+__device__ __forceinline__ void let_next_kernel_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 enum Mode { kSample = 0, kVerify = 1 };
 
@@ -114,6 +114,7 @@ struct Params {
   int extra;             // 1 when near-ties are counted: every race is run for one more arrival
   int top_cmax;          // cluster kernel for several arrivals: most arrivals any race of the call wants
   int top_split;         // the same kernel: 0, or 1 + the number of nodes with children when every row gets its own cluster
+  int early;             // cluster kernels: let the next kernel on the stream start early
   Slot* slots;
 };
 
@@ -642,6 +643,12 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   const size_t smem = (small ? b128::cluster_role_bytes<DT>(G, AL) : b256::cluster_role_bytes<DT>(G, AL)) * (size_t)roles +
                       (cmax > 1 ? b256::top_list_bytes(cmax, CL) : 0);
   Launch l(dim3((unsigned)CL, (unsigned)jobs, (unsigned)p.B), (unsigned)threads, smem, st, (unsigned)CL);
+  // The next kernel's blocks go where this one's leave room: if this one has a block on every SM they
+  // are spread unevenly when they start early.  (One row of 128256 logits 4.8 us with it and 5.0
+  // without, 4 x 8 alternatives 10.7 and 11.6, a tree of 240 blocks 21.1 and 22.1; but 16 rows, 256
+  // blocks, 9.1 and 8.1, 300 positions of 8192 logits 12.9 and 11.0, and the streaming kernel, two
+  // blocks to an SM, 47.5 and 38.9.)
+  p.early = (int64_t)CL * jobs * p.B <= (cmax > 1 ? 2 : 1) * sm_count();
   snprintf(g_last_launch, sizeof g_last_launch, "%s<%s, %d row(s) per cluster>: %d clusters of %d x %d threads, %d positions",
            cmax > 1 ? "ersd_cluster_top_kernel" : "ersd_cluster_kernel", DT == ERSD_BF16 ? "bf16" : "f32", roles,
            p.B * jobs, CL, threads, p.B * p.rows);
