@@ -455,24 +455,20 @@ static int launch(const Params& p, const TreeDesc& tree, int dt, int cmax, cudaS
 // ---------------------------------------------------------------------------------------------
 // Latency path of calls of few rows: one cluster of thread blocks per position (ersd_cluster.inc).
 // ---------------------------------------------------------------------------------------------
-// Default choice for races of one arrival, by the logits of the call (positions x V).  Short rows
-// always take the cluster kernel, longer ones up to a number of logits from which the streaming
-// kernel's throughput wins (measured with rows of eleven lengths from 1024 to 128256.  Verification,
-// bf16: at 16384 logits 800 positions take 34.3 us here and 37.5 streamed, 1200 48.6 and 46.8; at
-// 32000 200 positions 24.8 and 25.9, 300 30.0 and 29.4; at 128256 50 24.9 and 25.7, 100 39.4 and 34.5.
-// Sampling, one row per position: at 32000 1200 rows 52.5 and 55.2 us, at 128256 150 rows 30.0 and
-// 36.1, 200 39.6 and 38.6.  32-bit logits take twice the room: verification at 4096 logits 3200
-// positions 53.8 and 63.4 us, at 8192 400 23.7 and 23.2, at 32000 100 27.6 and 24.9; sampling at
-// 32000 100 rows 14.6 and 18.7, 400 38.2 and 26.9).
+// Default choice for races of one arrival, by the logits of the call (positions x V).  32-bit logits and
+// rows of up to about 40000 always take the cluster kernel (verification, cluster kernel / streaming
+// kernel: 6000 positions of 15048 bf16 logits 112.5 / 173 us, 2300 of 48000 120.9 / 134.5; 32-bit: 2000 of
+// 32000 92.1 / 148, 150 of 128256 39.6 / 60, 2300 of 151936 459 / 653; sampling of 2304 x 128256 256 /
+// 325).  The streaming kernel spends less on an index, once its thresholds have settled, and more on
+// starting: it takes longer bf16 rows from a number of logits on (verification: at 65256 logits 1200
+// positions 96.7 / 98.7 and 2000 144.8 / 143; at 128256 300 59.2 / 62.7 and 375 67.1 / 66.1, 600 101.8 /
+// 89.8; at 151936 250 56.4 / 58.8 and 400 81.4 / 76.4.  Sampling, one row per position: at 128256 800 93.1 / 95.1).
 struct ClusterLimit {
   int row;         // rows of up to this many logits ...
   int64_t logits;  // ... take the cluster kernel while the call has no more logits than this
 };
-constexpr ClusterLimit kClusterLimits[2][2][3] = {
-    // ERSD_F32: one row per position, draft and target row
-    {{{8192, INT64_MAX}, {16384, 18 << 20}, {INT32_MAX, 5 << 20}}, {{4096, INT64_MAX}, {8192, 8 << 20}, {INT32_MAX, 2 << 20}}},
-    // ERSD_BF16
-    {{{16384, INT64_MAX}, {32768, 36 << 20}, {INT32_MAX, 20 << 20}}, {{8192, INT64_MAX}, {16384, 16 << 20}, {INT32_MAX, 8 << 20}}}};
+constexpr ClusterLimit kClusterLimits[2][3] = {  // bf16: one row per position, draft and target row
+    {{65536, INT64_MAX}, {INT32_MAX, 100 << 20}}, {{49152, INT64_MAX}, {65536, 80 << 20}, {INT32_MAX, 40 << 20}}};
 // The same for races of several arrivals (ersd_cluster_top.inc; three blocks per SM).
 constexpr int64_t kClusterAutoBlocksTop = 600;
 // ... and the number of blocks up to which a tree's rows get a cluster each (one block per SM and a half)
@@ -498,13 +494,14 @@ static int cluster_limit(int* out) {
   if (dev < 0 || dev >= 64) return ERSD_EUNSUPPORTED;
   std::lock_guard<std::mutex> lock(m);
   if (!limit[dev]) {
-    constexpr int kKernels = 16, kSmall = 8;  // (the last kSmall: 128-thread blocks, never in clusters)
+    constexpr int kKernels = 24, kSmall = 8;  // (the last kSmall: 128-thread blocks, never in clusters)
     const void* kernels[kKernels + kSmall];
     int count = 0, small = kKernels;
     auto add = [&](auto dt, auto nr, auto al) {
-      kernels[count++] = (const void*)b256::ersd_cluster_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value>;
+      kernels[count++] = (const void*)b256::ersd_cluster_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value, true>;
       kernels[count++] = (const void*)b256::ersd_cluster_top_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value>;
-      kernels[small++] = (const void*)b128::ersd_cluster_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value>;
+      kernels[count++] = (const void*)b256::ersd_cluster_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value, false>;
+      kernels[small++] = (const void*)b128::ersd_cluster_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value, true>;
     };
     auto both = [&](auto dt, auto nr) {
       add(dt, nr, std::true_type());
@@ -589,6 +586,31 @@ static int cluster_size(const ersd_opts& o, const Params& p, int dt, int cmax, i
   return ERSD_OK;
 }
 
+// Races of one arrival: whether the call's logits are staged in shared memory.  Staged blocks have the
+// shortest path through a position but only two or three of them fit an SM; unstaged ones read the rows
+// tile by tile while they compute, four (of 128 threads: eight) to an SM, and fetch the few logits
+// they need again from L2.  Staged / unstaged us, verification of bf16 rows: 10 x 128256 logits 9.8 /
+// 10.4, 40 x 32000 9.7 / 10.2, 500 x 4096 11.0 / 11.3, 80 x 32000 13.2 / 12.3, 40 x 128256 22.2 / 15.9, 800
+// x 15048 32.5 / 25.8; sampling: 16 x 128256 8.0 / 8.6, 100 x 32000 9.1 / 9.0, 100 x 128256 21.8 /
+// 19.0; 32-bit: verification of 500 x 4096 14.1 / 12.2, sampling of 100 x 32000 12.6 / 8.8.
+constexpr int64_t kClusterStagedBytes = 8 << 20;
+static bool cluster_staged(const Params& p, int dt, int roles) {
+  return (int64_t)p.B * p.rows * p.V * (int64_t)elem_size(dt) * roles <= kClusterStagedBytes;
+}
+
+// Blocks per cluster, unstaged: as many as keep the call within about two blocks per SM (75 positions
+// of 128256 bf16 logits: 4 blocks 22.9 us, 8 24.7; 150 of 32000: 2 15.7, 4 19.0) while a block has at
+// least three tiles, and so many that it has no more than 16, which keeps the last wave short (300
+// positions of 128256: 1 block 111.6 us, 2 60.4, 4 57.2; 150 of 32-bit logits: 2 54.7, 4 39.5).
+static int unstaged_size(const Params& p, int dt, int roles, int lim) {
+  const int most = dt == ERSD_F32 && roles == 2 ? 20 : 32;
+  const int ntiles = (p.V + b256::kTile - 1) / b256::kTile;
+  const int64_t units = (int64_t)p.B * p.rows;
+  int CL = 1;
+  while (CL < lim && ((units * CL * 2 * 10 <= 22 * sm_count() && ntiles >= CL * 2 * 3) || ntiles > CL * most)) CL *= 2;
+  return CL;
+}
+
 // Whether a call that leaves the choice to the library takes the cluster kernel.
 static bool cluster_by_default(const ersd_opts& o, const Params& p, int dt, int cmax) {
   if (o.kernel_path != 0 || o.split_v != 0 || o.block_threads != 0 || !cluster_applies(p, dt, cmax)) return false;
@@ -596,7 +618,8 @@ static bool cluster_by_default(const ersd_opts& o, const Params& p, int dt, int 
   if (cluster_size(o, p, dt, cmax, &CL) != ERSD_OK) return false;
   const int64_t blocks = (int64_t)p.B * p.rows * CL;
   if (cmax > 1) return blocks <= kClusterAutoBlocksTop;
-  const ClusterLimit* limit = kClusterLimits[dt == ERSD_BF16][p.mode == kVerify && p.draft];
+  if (dt == ERSD_F32) return true;
+  const ClusterLimit* limit = kClusterLimits[p.mode == kVerify && p.draft];
   while (p.V > limit->row) ++limit;
   return (int64_t)p.V * p.B * p.rows <= limit->logits;
 }
@@ -635,12 +658,21 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   // instead of 25.0 us, verification 26.8 instead of 37.0; at 400 rows equal; blocks of 64 threads
   // 19.6 and 29.9), and for rows that 128 threads take in one turn (400 positions of 1024 logits: 8.4
   // instead of 10.4 us); not where the staged rows would leave fewer than five such blocks to an SM.
+  // Unstaged rows leave that room up to 16384 logits and beyond; longer ones keep 256 threads busy
+  // (800 positions of 15048 logits: 25.8 us with 128 threads, 27.0 with 256; 1200 of 32000 57.1 and 51.4).
+  const bool staged = cmax > 1 || cluster_staged(p, DT, roles);
+  if (!staged && !o.split_v) {
+    int lim = 8;
+    const int st2 = cluster_limit(&lim);
+    if (st2 != ERSD_OK) return st2;
+    CL = unstaged_size(p, DT, roles, lim);
+  }
   const int G128 = (p.V + b128::kTile - 1) / b128::kTile;
-  const bool small = cmax == 1 && CL == 1 && b128::cluster_role_bytes<DT>(G128, AL) * (size_t)roles <= 41 * 1024 &&
-                     ((int64_t)p.B * p.rows > 4 * sm_count() || G128 == 1);
+  const bool small = cmax == 1 && CL == 1 && ((int64_t)p.B * p.rows > 4 * sm_count() || G128 == 1) &&
+                     (staged ? b128::cluster_role_bytes<DT>(G128, AL) * (size_t)roles <= 41 * 1024 : G128 <= 16);
   const int threads = small ? b128::kThreads : b256::kThreads;
   const int G = small ? G128 : (ntiles + CL - 1) / CL;  // tiles per block; they fit, see cluster_applies
-  const size_t smem = (small ? b128::cluster_role_bytes<DT>(G, AL) : b256::cluster_role_bytes<DT>(G, AL)) * (size_t)roles +
+  const size_t smem = (small ? b128::cluster_role_bytes<DT>(G, AL, staged) : b256::cluster_role_bytes<DT>(G, AL, staged)) * (size_t)roles +
                       (cmax > 1 ? b256::top_list_bytes(cmax, CL) : 0);
   Launch l(dim3((unsigned)CL, (unsigned)jobs, (unsigned)p.B), (unsigned)threads, smem, st, (unsigned)CL);
   // The next kernel's blocks go where this one's leave room: if this one has a block on every SM they
@@ -649,16 +681,19 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   // blocks, 9.1 and 8.1, 300 positions of 8192 logits 12.9 and 11.0, and the streaming kernel, two
   // blocks to an SM, 47.5 and 38.9.)
   p.early = (int64_t)CL * jobs * p.B <= (cmax > 1 ? 2 : 1) * sm_count();
-  snprintf(g_last_launch, sizeof g_last_launch, "%s<%s, %d row(s) per cluster>: %d clusters of %d x %d threads, %d positions",
+  snprintf(g_last_launch, sizeof g_last_launch, "%s<%s, %d row(s) per cluster>%s: %d clusters of %d x %d threads, %d positions",
            cmax > 1 ? "ersd_cluster_top_kernel" : "ersd_cluster_kernel", DT == ERSD_BF16 ? "bf16" : "f32", roles,
-           p.B * jobs, CL, threads, p.B * p.rows);
+           staged ? "" : " (unstaged)", p.B * jobs, CL, threads, p.B * p.rows);
   cudaError_t e;
   if (cmax > 1) {
     auto kernel = roles == 2 ? b256::ersd_cluster_top_kernel<DT, 2, AL> : b256::ersd_cluster_top_kernel<DT, 1, AL>;
     e = cudaLaunchKernelEx(&l.cfg, kernel, p, tree);
   } else {
-    auto kernel = roles == 2 ? b256::ersd_cluster_kernel<DT, 2, AL> : b256::ersd_cluster_kernel<DT, 1, AL>;
-    if (small) kernel = roles == 2 ? b128::ersd_cluster_kernel<DT, 2, AL> : b128::ersd_cluster_kernel<DT, 1, AL>;
+    void (*kernel)(Params);
+    if (staged && small) kernel = roles == 2 ? b128::ersd_cluster_kernel<DT, 2, AL, true> : b128::ersd_cluster_kernel<DT, 1, AL, true>;
+    else if (staged) kernel = roles == 2 ? b256::ersd_cluster_kernel<DT, 2, AL, true> : b256::ersd_cluster_kernel<DT, 1, AL, true>;
+    else if (small) kernel = roles == 2 ? b128::ersd_cluster_kernel<DT, 2, AL, false> : b128::ersd_cluster_kernel<DT, 1, AL, false>;
+    else kernel = roles == 2 ? b256::ersd_cluster_kernel<DT, 2, AL, false> : b256::ersd_cluster_kernel<DT, 1, AL, false>;
     e = cudaLaunchKernelEx(&l.cfg, kernel, p);
   }
   return e == cudaSuccess ? ERSD_OK : cuda_fail(e);
