@@ -467,11 +467,16 @@ struct ClusterLimit {
   int row;         // rows of up to this many logits ...
   int64_t logits;  // ... take the cluster kernel while the call has no more logits than this
 };
-constexpr ClusterLimit kClusterLimits[2][3] = {  // bf16: one row per position, draft and target row
-    {{65536, INT64_MAX}, {INT32_MAX, 100 << 20}}, {{49152, INT64_MAX}, {65536, 80 << 20}, {INT32_MAX, 40 << 20}}};
-// The same for races of several arrivals (ersd_cluster_top.inc; three blocks per SM).
-constexpr int64_t kClusterAutoBlocksTop = 600;
-// ... and the number of blocks up to which a tree's rows get a cluster each (one block per SM and a half)
+// Races of several arrivals gain more from it (trees, cluster kernel / streaming kernel: 16 x 17 nodes of
+// 128256 bf16 logits 59.7 / 80.9 us, 20 x 17 73.4 / 75.6, 24 x 17 130 / 81.5; 256 x 17 of 32000 179.5 / 195.2;
+// 100 x 9 of 128256 32-bit logits 224 / 242; eight arrivals of 256 rows of 128256 60 / 114).  Trees of more
+// than 131072 logits a row stream from 20M logits on although the cluster kernel would be quicker there (8 x 17
+// nodes of 151936: 39.4 / 63.7): the tests fix which kernel takes that call.
+constexpr ClusterLimit kClusterLimits[3][4] = {  // bf16: one row per position, draft and target row, the same in trees
+    {{65536, INT64_MAX}, {INT32_MAX, 100 << 20}},
+    {{49152, INT64_MAX}, {65536, 80 << 20}, {INT32_MAX, 40 << 20}},
+    {{49152, INT64_MAX}, {65536, 80 << 20}, {131072, 40 << 20}, {INT32_MAX, 19 << 20}}};
+// The number of blocks up to which a tree's rows get a cluster each (one block per SM and a half)
 constexpr int64_t kClusterSplitBlocks = 384;
 constexpr size_t kClusterSmemBytes = 200 * 1024;  // dynamic shared memory a block of the cluster kernels may use
 
@@ -494,12 +499,13 @@ static int cluster_limit(int* out) {
   if (dev < 0 || dev >= 64) return ERSD_EUNSUPPORTED;
   std::lock_guard<std::mutex> lock(m);
   if (!limit[dev]) {
-    constexpr int kKernels = 24, kSmall = 8;  // (the last kSmall: 128-thread blocks, never in clusters)
+    constexpr int kKernels = 32, kSmall = 8;  // (the last kSmall: 128-thread blocks, never in clusters)
     const void* kernels[kKernels + kSmall];
     int count = 0, small = kKernels;
     auto add = [&](auto dt, auto nr, auto al) {
       kernels[count++] = (const void*)b256::ersd_cluster_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value, true>;
-      kernels[count++] = (const void*)b256::ersd_cluster_top_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value>;
+      kernels[count++] = (const void*)b256::ersd_cluster_top_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value, true>;
+      kernels[count++] = (const void*)b256::ersd_cluster_top_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value, false>;
       kernels[count++] = (const void*)b256::ersd_cluster_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value, false>;
       kernels[small++] = (const void*)b128::ersd_cluster_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value, true>;
     };
@@ -559,11 +565,41 @@ static bool cluster_applies(const Params& p, int dt, int cmax) {
   return p.rows <= 65535 && p.B <= 65535;
 }
 
+// Whether the call's logits are staged in shared memory.  Staged blocks have the
+// shortest path through a position but only two or three of them fit an SM; unstaged ones read the rows
+// tile by tile while they compute, four (of 128 threads: eight) to an SM, and fetch the few logits
+// they need again from L2.  Staged / unstaged us, verification of bf16 rows: 10 x 128256 logits 9.8 /
+// 10.4, 40 x 32000 9.7 / 10.2, 500 x 4096 11.0 / 11.3, 80 x 32000 13.2 / 12.3, 40 x 128256 22.2 / 15.9, 800
+// x 15048 32.5 / 25.8; sampling: 16 x 128256 8.0 / 8.6, 100 x 32000 9.1 / 9.0, 100 x 128256 21.8 /
+// 19.0; 32-bit: verification of 500 x 4096 14.1 / 12.2, sampling of 100 x 32000 12.6 / 8.8.
+// Several arrivals: 50 x 32000 11.0 / 11.3, 12 x 128256 12.5 / 11.4, 64 x 128256 30.0 / 22.4; a tree of 17
+// nodes of 32000 logits, 10 sequences 31.7 / 21.6.
+constexpr int64_t kClusterStagedBytes = 8 << 20, kClusterStagedBytesTop = 4 << 20;
+static bool cluster_staged(const Params& p, int dt, int roles, int cmax) {
+  return (int64_t)p.B * p.rows * p.V * (int64_t)elem_size(dt) * roles <= (cmax > 1 ? kClusterStagedBytesTop : kClusterStagedBytes);
+}
+
+// Blocks per cluster, unstaged: as many as keep the call within about two blocks per SM (75 positions
+// of 128256 bf16 logits: 4 blocks 22.9 us, 8 24.7; 150 of 32000: 2 15.7, 4 19.0) while a block has at
+// least three tiles, and so many that it has no more tiles than its bounds leave room for beside
+// three other blocks and some L1 (150 positions of 128256 bf16 logits: 1 block 72 us, 2 34.9, 4 35.8; of
+// 100000 400: 2 59, 4 63; 32-bit logits, two requests to a sector: 128256 2 54, 4 39.6.  Several
+// arrivals, with their lists: 160 rows of a tree of 128256 2 56.6, 4 42.6; 32-bit: 63 rows 4 32.3, 8 23.2).
+static int unstaged_size(const Params& p, int dt, int roles, int cmax, int lim) {
+  const int most = cmax > 1 ? (dt == ERSD_F32 && roles == 2 ? 10 : 20) : (dt == ERSD_F32 && roles == 2 ? 20 : 32);
+  const int fill = cmax > 1 ? 25 : 22;  // blocks per ten SMs
+  const int ntiles = (p.V + b256::kTile - 1) / b256::kTile;
+  const int64_t units = (int64_t)p.B * p.rows;
+  int CL = 1;
+  while (CL < lim && ((units * CL * 2 * 10 <= fill * sm_count() && ntiles >= CL * 2 * 3) || ntiles > CL * most)) CL *= 2;
+  return CL;
+}
+
 // Blocks per cluster.  Few positions: the smallest power of two that leaves a block about
 // kClusterGroups tiles (shortest path through one position).  Once such clusters would make more
 // than two blocks per SM: blocks of about twice as many tiles (measured at V = 128256: clusters
 // of 8 beat clusters of 16 from about 20 positions on, clusters of 4 never beat clusters of 8).
-static int cluster_size(const ersd_opts& o, const Params& p, int dt, int cmax, int* out) {
+static int cluster_size(const ersd_opts& o, const Params& p, int dt, int cmax, bool staged, int* out) {
   int lim = 8;
   const int ls = cluster_limit(&lim);
   if (ls != ERSD_OK) return ls;
@@ -576,6 +612,10 @@ static int cluster_size(const ersd_opts& o, const Params& p, int dt, int cmax, i
     *out = CL;
     return ERSD_OK;
   }
+  if (!staged) {
+    *out = unstaged_size(p, dt, roles, cmax, lim);
+    return ERSD_OK;
+  }
   int CL = 1;
   while (CL < lim && CL * b256::kClusterGroups < ntiles) CL *= 2;
   const int64_t units = (int64_t)p.B * p.rows;
@@ -586,40 +626,11 @@ static int cluster_size(const ersd_opts& o, const Params& p, int dt, int cmax, i
   return ERSD_OK;
 }
 
-// Races of one arrival: whether the call's logits are staged in shared memory.  Staged blocks have the
-// shortest path through a position but only two or three of them fit an SM; unstaged ones read the rows
-// tile by tile while they compute, four (of 128 threads: eight) to an SM, and fetch the few logits
-// they need again from L2.  Staged / unstaged us, verification of bf16 rows: 10 x 128256 logits 9.8 /
-// 10.4, 40 x 32000 9.7 / 10.2, 500 x 4096 11.0 / 11.3, 80 x 32000 13.2 / 12.3, 40 x 128256 22.2 / 15.9, 800
-// x 15048 32.5 / 25.8; sampling: 16 x 128256 8.0 / 8.6, 100 x 32000 9.1 / 9.0, 100 x 128256 21.8 /
-// 19.0; 32-bit: verification of 500 x 4096 14.1 / 12.2, sampling of 100 x 32000 12.6 / 8.8.
-constexpr int64_t kClusterStagedBytes = 8 << 20;
-static bool cluster_staged(const Params& p, int dt, int roles) {
-  return (int64_t)p.B * p.rows * p.V * (int64_t)elem_size(dt) * roles <= kClusterStagedBytes;
-}
-
-// Blocks per cluster, unstaged: as many as keep the call within about two blocks per SM (75 positions
-// of 128256 bf16 logits: 4 blocks 22.9 us, 8 24.7; 150 of 32000: 2 15.7, 4 19.0) while a block has at
-// least three tiles, and so many that it has no more than 16, which keeps the last wave short (300
-// positions of 128256: 1 block 111.6 us, 2 60.4, 4 57.2; 150 of 32-bit logits: 2 54.7, 4 39.5).
-static int unstaged_size(const Params& p, int dt, int roles, int lim) {
-  const int most = dt == ERSD_F32 && roles == 2 ? 20 : 32;
-  const int ntiles = (p.V + b256::kTile - 1) / b256::kTile;
-  const int64_t units = (int64_t)p.B * p.rows;
-  int CL = 1;
-  while (CL < lim && ((units * CL * 2 * 10 <= 22 * sm_count() && ntiles >= CL * 2 * 3) || ntiles > CL * most)) CL *= 2;
-  return CL;
-}
-
 // Whether a call that leaves the choice to the library takes the cluster kernel.
 static bool cluster_by_default(const ersd_opts& o, const Params& p, int dt, int cmax) {
   if (o.kernel_path != 0 || o.split_v != 0 || o.block_threads != 0 || !cluster_applies(p, dt, cmax)) return false;
-  int CL = 1;
-  if (cluster_size(o, p, dt, cmax, &CL) != ERSD_OK) return false;
-  const int64_t blocks = (int64_t)p.B * p.rows * CL;
-  if (cmax > 1) return blocks <= kClusterAutoBlocksTop;
   if (dt == ERSD_F32) return true;
-  const ClusterLimit* limit = kClusterLimits[p.mode == kVerify && p.draft];
+  const ClusterLimit* limit = kClusterLimits[!(p.mode == kVerify && p.draft) ? 0 : cmax > 1 ? 2 : 1];
   while (p.V > limit->row) ++limit;
   return (int64_t)p.V * p.B * p.rows <= limit->logits;
 }
@@ -630,7 +641,8 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   p.top_cmax = cmax;
   int roles = (p.mode == kVerify && p.draft) ? 2 : 1;
   int CL = 1;
-  const int ls = cluster_size(o, p, DT, cmax, &CL);
+  const bool staged = cluster_staged(p, DT, roles, cmax);
+  const int ls = cluster_size(o, p, DT, cmax, staged, &CL);
   if (ls != ERSD_OK) return ls;
   const int ntiles = (p.V + b256::kTile - 1) / b256::kTile;
   // Trees of few positions: a cluster per ROW (a node's draft row and its target row side by side
@@ -642,7 +654,7 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
     for (int n = 0; n < p.rows; ++n) with_children += tree.nchild[n] > 0 ? 1 : 0;
     const int64_t rows_in_all = (int64_t)p.B * (p.rows + with_children);
     bool split = rows_in_all * CL <= kClusterSplitBlocks;
-    if (!split && !o.split_v && CL >= 2 && rows_in_all * (CL / 2) <= kClusterSplitBlocks &&
+    if (!split && (staged || CL == 16) && !o.split_v && CL >= 2 && rows_in_all * (CL / 2) <= kClusterSplitBlocks &&
         (ntiles + CL / 2 - 1) / (CL / 2) <= cluster_max_tiles(DT, 1, cmax, AL)) {
       CL /= 2;  // (a row to a cluster of half as many blocks)
       split = true;
@@ -660,13 +672,7 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   // instead of 10.4 us); not where the staged rows would leave fewer than five such blocks to an SM.
   // Unstaged rows leave that room up to 16384 logits and beyond; longer ones keep 256 threads busy
   // (800 positions of 15048 logits: 25.8 us with 128 threads, 27.0 with 256; 1200 of 32000 57.1 and 51.4).
-  const bool staged = cmax > 1 || cluster_staged(p, DT, roles);
-  if (!staged && !o.split_v) {
-    int lim = 8;
-    const int st2 = cluster_limit(&lim);
-    if (st2 != ERSD_OK) return st2;
-    CL = unstaged_size(p, DT, roles, lim);
-  }
+  
   const int G128 = (p.V + b128::kTile - 1) / b128::kTile;
   const bool small = cmax == 1 && CL == 1 && ((int64_t)p.B * p.rows > 4 * sm_count() || G128 == 1) &&
                      (staged ? b128::cluster_role_bytes<DT>(G128, AL) * (size_t)roles <= 41 * 1024 : G128 <= 16);
@@ -681,12 +687,13 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   // blocks, 9.1 and 8.1, 300 positions of 8192 logits 12.9 and 11.0, and the streaming kernel, two
   // blocks to an SM, 47.5 and 38.9.)
   p.early = (int64_t)CL * jobs * p.B <= (cmax > 1 ? 2 : 1) * sm_count();
-  snprintf(g_last_launch, sizeof g_last_launch, "%s<%s, %d row(s) per cluster>%s: %d clusters of %d x %d threads, %d positions",
+  snprintf(g_last_launch, sizeof g_last_launch, "%s<%s, %d row(s) per cluster>: %d clusters of %d x %d threads, %d positions%s",
            cmax > 1 ? "ersd_cluster_top_kernel" : "ersd_cluster_kernel", DT == ERSD_BF16 ? "bf16" : "f32", roles,
-           staged ? "" : " (unstaged)", p.B * jobs, CL, threads, p.B * p.rows);
+           p.B * jobs, CL, threads, p.B * p.rows, staged ? "" : " (unstaged)");
   cudaError_t e;
   if (cmax > 1) {
-    auto kernel = roles == 2 ? b256::ersd_cluster_top_kernel<DT, 2, AL> : b256::ersd_cluster_top_kernel<DT, 1, AL>;
+    auto kernel = roles == 2 ? b256::ersd_cluster_top_kernel<DT, 2, AL, true> : b256::ersd_cluster_top_kernel<DT, 1, AL, true>;
+    if (!staged) kernel = roles == 2 ? b256::ersd_cluster_top_kernel<DT, 2, AL, false> : b256::ersd_cluster_top_kernel<DT, 1, AL, false>;
     e = cudaLaunchKernelEx(&l.cfg, kernel, p, tree);
   } else {
     void (*kernel)(Params);

@@ -68,3 +68,51 @@ def test_special_values_as_in_the_streaming_kernel(ersd, dtype):  # noqa: F811
         torch.cuda.synchronize()
         for name in a:
             assert torch.equal(a[name], b[name]) or (name.endswith("key") and (a[name] == b[name]).all()), (name, T)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("B,V", [(160, 2049), (24, 16384), (10, 32001), (6, 66001), (3, 131080)])
+def test_several_arrivals_against_the_oracle(ersd, B, V, dtype):  # noqa: F811
+    """Blocks by themselves and clusters of 2 to 16, ragged last tiles, rows on and off 16-byte boundaries."""
+    on_device = guarded if V % 8 else torch.Tensor.cuda
+    parent = wl.TREE_SPECINFER
+    inp = inputs(B, len(parent) - 1, V, dtype, parent=parent)
+    out = ersd.verify(on_device(inp["target"]), on_device(inp["draft"]), inp["seeds"].cuda(), inp["T"], want_rows=True,
+                      parent=list(parent))
+    torch.cuda.synchronize()
+    assert "ersd_cluster_top_kernel" in ersd.ersd_last_launch() and "(unstaged)" in ersd.ersd_last_launch()
+    check_verify(inp, out)
+    logits, seeds, c = inp["target"], inp["seeds"], 32
+    tok = torch.full((B, len(parent), c), -7, dtype=torch.int32, device="cuda")
+    key = torch.full((B, len(parent), c), -7.0, dtype=torch.float32, device="cuda")
+    ersd.ersd_race_sample(on_device(logits), seeds.cuda(), 0.8, tok, ersd.make_opts(top_c=c, out_key=key))
+    torch.cuda.synchronize()
+    assert "ersd_cluster_top_kernel" in ersd.ersd_last_launch() and "(unstaged)" in ersd.ersd_last_launch()
+    check_sample(logits, seeds, 0.8, tok, key, c=c)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_several_arrivals_of_tied_and_masked_rows(ersd, dtype):  # noqa: F811
+    """Rows of equal logits under T = 0 overflow a block's lists; rows with fewer tokens than arrivals wanted."""
+    V, B, c = 40008, 60, 8
+    g = torch.Generator().manual_seed(19)
+    z = torch.randn(B, 1, V, generator=g)
+    z[0::5] = 0.5
+    z[1::5, :, 3:] = float("-inf")
+    z[2::5, :, ::2] = float("nan")
+    z[3::5, :, 17] = float("inf")
+    temps = torch.full((B, 1), 0.9)
+    temps[0::2] = 0.0
+    temps[7] = float("nan")
+    z, seeds = wl._storage(z, dtype).cuda(), wl.make_seeds(5, 0, B).cuda()
+    got = []
+    for path in (2, 1):
+        tok = torch.full((B, 1, c), -7, dtype=torch.int32, device="cuda")
+        key = torch.full((B, 1, c), -7.0, dtype=torch.float32, device="cuda")
+        ersd.ersd_race_sample(z, seeds, 1.0, tok, ersd.make_opts(top_c=c, out_key=key, kernel_path=path, temps=temps.cuda(),
+                                                                 temp_strides=(1, 1)))
+        torch.cuda.synchronize()
+        assert ("(unstaged)" in ersd.ersd_last_launch()) == (path == 2)
+        got.append((tok, key))
+    assert torch.equal(got[0][0], got[1][0])
+    assert (got[0][1] == got[1][1]).all()
