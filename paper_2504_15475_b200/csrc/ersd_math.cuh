@@ -25,6 +25,24 @@ ERSD_HD void mulhilo(uint32_t a, uint32_t b, uint32_t& hi, uint32_t& lo) {
   lo = (uint32_t)p;
 }
 
+// The same product in two instructions, one per half.  The wide multiply wants its result in an even
+// register pair, which costs moves and registers where the halves part company at once: the loop of the
+// unstaged cluster kernel runs 4 % quicker with two (150 positions of 32000 bf16 logits 15.7 -> 14.9 us, 150
+// of 128256 34.2 -> 32.8), that of the streaming kernel 0.4 % slower.
+ERSD_HD void mulhilo_split(uint32_t a, uint32_t b, uint32_t& hi, uint32_t& lo) {
+#if defined(__CUDA_ARCH__)
+  hi = __umulhi(a, b);
+  asm("mul.lo.u32 %0, %1, %2;" : "=r"(lo) : "r"(a), "r"(b));
+#else
+  mulhilo(a, b, hi, lo);
+#endif
+}
+template <bool SPLIT>
+ERSD_HD void product(uint32_t a, uint32_t b, uint32_t& hi, uint32_t& lo) {
+  if (SPLIT) mulhilo_split(a, b, hi, lo);
+  else mulhilo(a, b, hi, lo);
+}
+
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds of two
 // 32x32->64 products and a word shuffle, the key advancing by the Weyl
 // constants between rounds.
@@ -60,6 +78,7 @@ struct PhiloxRow {
   uint32_t r3_b;         // round 3: c2' = hi(M0*c0) ^ r3_b             (r3_b = lo(M0*A0) ^ k1[2])
   uint32_t k0[10], k1[10];  // round keys (entries 2.. / 3.. are used)
 
+  template <bool SPLIT = false>
   ERSD_HD void init(uint64_t seed, uint32_t seq_id, uint32_t position, uint32_t stream = 0) {
     uint32_t a = (uint32_t)seed, b = (uint32_t)(seed >> 32);
 #pragma unroll
@@ -70,30 +89,31 @@ struct PhiloxRow {
       b += kPhiloxW1;
     }
     uint32_t hi1, lo1, H0, L0;
-    mulhilo(kPhiloxM1, seq_id, hi1, lo1);
+    product<SPLIT>(kPhiloxM1, seq_id, hi1, lo1);
     const uint32_t A0 = hi1 ^ position ^ k0[0];  // c0 after round 1
-    mulhilo(kPhiloxM0, A0, H0, L0);
+    product<SPLIT>(kPhiloxM0, A0, H0, L0);
     r1_k1 = stream ^ k1[0];
     r2_a = lo1 ^ k0[1];
     r2_b = H0 ^ k1[1];
     r3_b = L0 ^ k1[2];
   }
 
+  template <bool SPLIT = false>
   ERSD_HD void words(uint32_t c0, uint32_t out[4]) const {
     uint32_t hi0, lo0, hi1, lo1;
-    mulhilo(kPhiloxM0, c0, hi0, lo0);  // round 1
+    product<SPLIT>(kPhiloxM0, c0, hi0, lo0);  // round 1
     uint32_t c2 = hi0 ^ r1_k1, c3 = lo0;
-    mulhilo(kPhiloxM1, c2, hi1, lo1);  // round 2
+    product<SPLIT>(kPhiloxM1, c2, hi1, lo1);  // round 2
     uint32_t n0 = hi1 ^ r2_a, n1 = lo1, n2 = c3 ^ r2_b;
-    mulhilo(kPhiloxM0, n0, hi0, lo0);  // round 3
-    mulhilo(kPhiloxM1, n2, hi1, lo1);
+    product<SPLIT>(kPhiloxM0, n0, hi0, lo0);  // round 3
+    product<SPLIT>(kPhiloxM1, n2, hi1, lo1);
     uint32_t c0v = hi1 ^ n1 ^ k0[2], c1 = lo1;
     c2 = hi0 ^ r3_b;
     c3 = lo0;
 #pragma unroll
     for (int r = 3; r < 10; ++r) {
-      mulhilo(kPhiloxM0, c0v, hi0, lo0);
-      mulhilo(kPhiloxM1, c2, hi1, lo1);
+      product<SPLIT>(kPhiloxM0, c0v, hi0, lo0);
+      product<SPLIT>(kPhiloxM1, c2, hi1, lo1);
       c0v = hi1 ^ c1 ^ k0[r];
       c1 = lo1;
       c2 = hi0 ^ c3 ^ k1[r];
