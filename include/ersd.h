@@ -28,9 +28,9 @@
  *     owned by the caller; the library never frees or keeps caller memory.
  *   - Logit tensors are row-major with the vocabulary contiguous.  Rows are
  *     `ld` elements apart (opts->ld_*; 0 means V) and row (b, r) starts at
- *     element (b * rows_per_sequence + r) * ld.  16-byte aligned rows take
- *     the vectorised path; other alignments are accepted and take a slower
- *     scalar path.
+ *     element (b * rows_per_sequence + r) * ld.  Rows of any alignment are
+ *     read sixteen bytes at a time; those off a 16-byte boundary cost a
+ *     shift of each group of eight logits, 5 to 25 % of a call's time.
  *   - Calls are asynchronous on `cuda_stream` (a cudaStream_t, NULL = default
  *     stream) and never synchronise.  The return value is a host-side status:
  *     argument errors are found before anything is launched, launch errors
@@ -112,11 +112,10 @@ typedef struct ersd_opts {
   uint32_t kernel_path;    /* ersd_race_sample, ersd_verify, ersd_verify_tokens, ersd_verify_noalloc,
                               ersd_verify_tree:
                               0 = chosen by the library, 1 = the streaming kernel, 2 = a cluster kernel
-                              (one thread-block cluster per position, for calls of few rows; one kernel for
-                              races of one arrival, one for races of up to 32: top_c > 1, trees with
-                              branching;
+                              (one thread-block cluster per position; one kernel for races of one arrival, one
+                              for races of up to 32: top_c > 1, trees with branching;
                               ERSD_EUNSUPPORTED where neither applies: a race of more than 32 arrivals,
-                              rows not 16-byte aligned, B or R > 65535, more than 32 rows per sequence
+                              rows not 16-byte aligned (the library's own choice takes those too), B or R > 65535, more than 32 rows per sequence
                               in ersd_verify and its variants, near_tie_count given, or a vocabulary too
                               long for eight blocks to stage in shared memory: beyond about 320 k entries
                               in bf16, 160 k in fp32, halved when draft rows are raced along, less the

@@ -453,7 +453,7 @@ static int launch(const Params& p, const TreeDesc& tree, int dt, int cmax, cudaS
 }
 
 // ---------------------------------------------------------------------------------------------
-// Latency path of calls of few rows: one cluster of thread blocks per position (ersd_cluster.inc).
+// One cluster of thread blocks per position (ersd_cluster.inc, ersd_cluster_top.inc).
 // ---------------------------------------------------------------------------------------------
 // Default choice for races of one arrival, by the logits of the call (positions x V).  32-bit logits and
 // rows of up to about 40000 always take the cluster kernel (verification, cluster kernel / streaming
@@ -1157,6 +1157,6 @@ int ersd_last_cuda_error(void) { return g_last_cuda_error; }
 
 const char* ersd_last_launch(void) { return g_last_launch; }
 
-int ersd_version(void) { return 111; }
+int ersd_version(void) { return 112; }
 
 }  // extern "C"
