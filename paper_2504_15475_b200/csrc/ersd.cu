@@ -579,19 +579,20 @@ static bool cluster_staged(const Params& p, int dt, int roles, int cmax) {
   return (int64_t)p.B * p.rows * p.V * (int64_t)elem_size(dt) * roles <= (cmax > 1 ? kClusterStagedBytesTop : kClusterStagedBytes);
 }
 
-// Blocks per cluster, unstaged: as many as keep the call within about two blocks per SM (75 positions
-// of 128256 bf16 logits: 4 blocks 22.9 us, 8 24.7; 150 of 32000: 2 15.7, 4 19.0) while a block has at
-// least three tiles, and so many that it has no more tiles than its bounds leave room for beside
+// Blocks per cluster, unstaged: a power of two (clusters of 3, 5, 6 or 7 were measured too: rarely the best,
+// never by more than 7 %), as large as keeps the call a little within the four blocks an SM takes, so that no
+// cluster waits for room (200 positions of 32000 bf16 logits: 1 block 19.6 us, 2 16.3; 100 of 128256: 2 31.0, 4
+// 23.2; 272 rows of trees of 32000: 1 27.5, 2 24.5; but 75 of 128256, 600 blocks: 4 22.3, 8 23.8, and 150 of
+// 32000: 2 15.1, 4 18.3) while a block has at least four tiles (250 of 12288: 1 block 12.9, 2 13.8), and so many that it has no more tiles than its bounds leave room for beside
 // three other blocks and some L1 (150 positions of 128256 bf16 logits: 1 block 72 us, 2 34.9, 4 35.8; of
 // 100000 400: 2 59, 4 63; 32-bit logits, two requests to a sector: 128256 2 54, 4 39.6.  Several
 // arrivals, with their lists: 160 rows of a tree of 128256 2 56.6, 4 42.6; 32-bit: 63 rows 4 32.3, 8 23.2).
 static int unstaged_size(const Params& p, int dt, int roles, int cmax, int lim) {
   const int most = cmax > 1 ? (dt == ERSD_F32 && roles == 2 ? 10 : 20) : (dt == ERSD_F32 && roles == 2 ? 20 : 32);
-  const int fill = cmax > 1 ? 25 : 22;  // blocks per ten SMs
   const int ntiles = (p.V + b256::kTile - 1) / b256::kTile;
   const int64_t units = (int64_t)p.B * p.rows;
   int CL = 1;
-  while (CL < lim && ((units * CL * 2 * 10 <= fill * sm_count() && ntiles >= CL * 2 * 3) || ntiles > CL * most)) CL *= 2;
+  while (CL < lim && ((units * CL * 2 * 10 <= 37 * sm_count() && ntiles >= CL * 2 * 4) || ntiles > CL * most)) CL *= 2;
   return CL;
 }
 
