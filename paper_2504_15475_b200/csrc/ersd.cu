@@ -456,13 +456,13 @@ static int launch(const Params& p, const TreeDesc& tree, int dt, int cmax, cudaS
 // One cluster of thread blocks per position (ersd_cluster.inc, ersd_cluster_top.inc).
 // ---------------------------------------------------------------------------------------------
 // Default choice for races of one arrival, by the logits of the call (positions x V).  32-bit logits and
-// rows of up to about 40000 always take the cluster kernel (verification, cluster kernel / streaming
+// rows of up to 65536 always take the cluster kernel (verification, cluster kernel / streaming
 // kernel: 6000 positions of 15048 bf16 logits 112.5 / 173 us, 2300 of 48000 120.9 / 134.5; 32-bit: 2000 of
 // 32000 92.1 / 148, 150 of 128256 39.6 / 60, 2300 of 151936 459 / 653; sampling of 2304 x 128256 256 /
 // 325).  The streaming kernel spends less on an index, once its thresholds have settled, and more on
-// starting: it takes longer bf16 rows from a number of logits on (verification: at 65256 logits 1200
-// positions 96.7 / 98.7 and 2000 144.8 / 143; at 128256 300 59.2 / 62.7 and 375 67.1 / 66.1, 600 101.8 /
-// 89.8; at 151936 250 56.4 / 58.8 and 400 81.4 / 76.4.  Sampling, one row per position: at 128256 800 93.1 / 95.1).
+// starting: it takes longer bf16 rows from a number of logits on (verification: at 65256 logits 1500
+// positions 111.2 / 113.5 and 2250 157.2 / 159.5; at 100000 500 65.5 / 69.7; at 128256 400 66.4 / 68.8, 450
+// 77.9 / 81.0, 576 91.8 / 87.5; at 151936 300 64.0 / 71.4 and 400 81.4 / 76.4; trees: at 128256 450 rows 85.7 / 83.8.  Sampling, one row per position: at 128256 800 93.1 / 95.1).
 struct ClusterLimit {
   int row;         // rows of up to this many logits ...
   int64_t logits;  // ... take the cluster kernel while the call has no more logits than this
@@ -474,7 +474,7 @@ struct ClusterLimit {
 // nodes of 151936: 39.4 / 63.7): the tests fix which kernel takes that call.
 constexpr ClusterLimit kClusterLimits[3][4] = {  // bf16: one row per position, draft and target row, the same in trees
     {{65536, INT64_MAX}, {INT32_MAX, 100 << 20}},
-    {{49152, INT64_MAX}, {65536, 80 << 20}, {INT32_MAX, 40 << 20}},
+    {{65536, INT64_MAX}, {INT32_MAX, 56 << 20}},
     {{49152, INT64_MAX}, {65536, 80 << 20}, {131072, 40 << 20}, {INT32_MAX, 19 << 20}}};
 // The number of blocks up to which a tree's rows get a cluster each (one block per SM and a half)
 constexpr int64_t kClusterSplitBlocks = 384;
