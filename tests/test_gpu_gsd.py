@@ -243,3 +243,30 @@ def test_final_races_too_close_for_single_precision(ersd):
     ersd.ersd_gsd_verify(tgt.cuda(), None, None, seeds.cuda(), 1.0, out, acc)
     torch.cuda.synchronize()
     assert (acc == 0).all() and (out.cpu().numpy()[ok] == ref["tokens"][ok]).all()
+
+
+def test_long_drafts_that_end_in_exact_races(ersd):
+    """More output columns than a warp has lanes, races decided by single and by double precision in
+    neighbouring sequences: the last block of every sequence writes all its columns and leaves all of
+    its scratch zeroed."""
+    B, k, V = 48, 40, 600
+    w = wl.Workload("gsdlong", B=B, k=k, V=V, dtype="f32", sigma=0.0, T=1.0, config_id=52)
+    inp = wl.make_inputs(w)
+    tok = draft_tokens(ersd, inp["draft"].cuda(), inp["seeds"].cuda(), inp["T"])[..., 0].contiguous()
+    for b in range(0, B, 2):                                    # a law without support ends every other sequence
+        inp["target"][b, (7 * b) % (k + 1)] = float("-inf")
+    ref = oracle.gsd_verify(wl.as_numpy_logits(inp["target"]), wl.as_numpy_logits(inp["draft"]), tok.cpu().numpy(),
+                            wl.seeds_as_u64(inp["seeds"]), T=inp["T"])
+    ok = ~ambiguous(ref)
+    assert ok.sum() >= B - 1 and (ref["accept_len"] == k).sum() >= B // 4
+    tgt, drf, seeds = inp["target"].cuda(), inp["draft"].cuda(), inp["seeds"].cuda()
+    ws = torch.empty(ersd.ersd_workspace_bytes(B, k + 1), dtype=torch.uint8, device="cuda")
+    ersd.ersd_workspace_init(ws)
+    for rep in range(5):
+        out = torch.full((B, k + 1), -9, dtype=torch.int32, device="cuda")
+        acc = torch.full((B,), -9, dtype=torch.int32, device="cuda")
+        ersd.ersd_gsd_verify(tgt, drf, tok, seeds, inp["T"], out, acc, ersd.make_opts(workspace=ws))
+        torch.cuda.synchronize()
+        assert (ws == 0).all(), rep
+        assert (acc.cpu().numpy()[ok] == ref["accept_len"][ok]).all()
+        assert (out.cpu().numpy()[ok] == ref["tokens"][ok]).all()
