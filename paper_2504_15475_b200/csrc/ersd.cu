@@ -182,8 +182,11 @@ __global__ void ersd_row_keys_kernel(const void* row, int V, float T, uint64_t s
 static thread_local int g_last_cuda_error = 0;
 static thread_local char g_last_launch[160] = "";  // ersd_last_launch(): what this thread's last call launched
 
+// The error stays with the library: the runtime keeps it per thread too, where the next check of some
+// other launch on this thread would find it.
 static int cuda_fail(cudaError_t e) {
   g_last_cuda_error = (int)e;
+  (void)cudaGetLastError();
   return ERSD_ECUDA;
 }
 
