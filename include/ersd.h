@@ -236,7 +236,8 @@ int ersd_verify_tokens(const void* target_logits, const int32_t* draft_tokens, e
  *   out_accept_len device [B] int32
  * opts: ld_*, temps (every temperature must be > 0), seq_ids, pos_offsets,
  * workspace (ersd_workspace_bytes(B, k + 1) bytes, as for ersd_verify; left zeroed).
- * Errors as for ersd_verify; T <= 0 is ERSD_EINVAL (the test needs a softmax).
+ * Errors as for ersd_verify; T <= 0 is ERSD_EINVAL (the test needs a softmax), B > 65535
+ * ERSD_EUNSUPPORTED (the launch grid's second dimension).
  */
 int ersd_gsd_verify(const void* target_logits, const void* draft_logits, const int32_t* draft_tokens,
                     ersd_dtype dt, const uint64_t* seeds, int B, int k, int V, float T, int32_t* out_tokens,

@@ -1061,6 +1061,7 @@ int ersd_gsd_verify(const void* target_logits, const void* draft_logits, const i
   gsd_fill(g, o, target_logits, draft_logits, draft_tokens, seeds, B, k, V, T, k + 1, k, out_tokens,
            out_accept_len);
   if (g.ld_t < V || g.ld_d < V) return ERSD_EINVAL;
+  if (B > 65535) return ERSD_EUNSUPPORTED;  // (sequences are the second dimension of both grids)
   // Sums: about 64 warps per multiprocessor in all, two waves of the 32 that are resident (32 or 128
   // per multiprocessor: 1 and 4 % slower at 64 sequences of 128256 logits).  Race: one wave of three
   // blocks per multiprocessor, because a block begins with the ratio tests.
@@ -1078,7 +1079,11 @@ int ersd_gsd_verify(const void* target_logits, const void* draft_logits, const i
   const bool bf16 = dt == ERSD_BF16;
   Launch sums(sums_grid, kGsdStatsThreads, 0, stream), race(race_grid, kGsdThreads, 0, stream);
   cudaError_t e = cudaLaunchKernelEx(&sums.cfg, bf16 ? gsd_stats_kernel<ERSD_BF16> : gsd_stats_kernel<ERSD_F32>, g);
-  if (e == cudaSuccess) e = cudaLaunchKernelEx(&race.cfg, bf16 ? gsd_race_kernel<ERSD_BF16> : gsd_race_kernel<ERSD_F32>, g);
+  if (e == cudaSuccess) {
+    e = cudaLaunchKernelEx(&race.cfg, bf16 ? gsd_race_kernel<ERSD_BF16> : gsd_race_kernel<ERSD_F32>, g);
+    // (the sums are on their way and nobody will clear them)
+    if (e != cudaSuccess) (void)cudaMemsetAsync(ws, 0, workspace_bytes(B, k + 1), stream);
+  }
   return e == cudaSuccess ? ERSD_OK : cuda_fail(e);
 }
 
