@@ -111,7 +111,7 @@ def native():
                                % (__file__, e)) from None
         _ersd_call.use(*[C.cast(f, C.c_void_p).value for f in (
             L.ersd_race_sample, L.ersd_verify, L.ersd_verify_noalloc, L.ersd_verify_tokens, L.ersd_verify_tree,
-            L.ersd_gsd_verify, L.ersd_gsd_verify_tree)])
+            L.ersd_gsd_verify, L.ersd_gsd_verify_tree)], ErsdOpts)
         _native = _ersd_call
     return _native
 

@@ -22,6 +22,8 @@ decltype(&ersd_verify_tree) f_verify_tree;
 decltype(&ersd_gsd_verify) f_gsd_verify;
 decltype(&ersd_gsd_verify_tree) f_gsd_verify_tree;
 
+PyObject* options_type;  // binding.py's ErsdOpts
+
 struct Failed {};  // a Python exception is set
 
 const char* dtype_name(at::ScalarType t) {
@@ -126,16 +128,23 @@ void* stream_of(PyObject* o) {
   return p;
 }
 
-// The options structure (a ctypes structure, which lends its memory), or none.
+// The options structure (an ErsdOpts, which lends its memory), or none.  Nothing else is taken: the
+// library copies the whole structure, addresses and all.
 struct Options {
   Py_buffer view;
   const ersd_opts* ptr = nullptr;
   explicit Options(PyObject* o) {
     if (o == Py_None) return;
+    const int is_options = PyObject_IsInstance(o, options_type);
+    if (is_options < 0) throw Failed();
+    if (!is_options) {
+      PyErr_Format(PyExc_TypeError, "opts must be an ErsdOpts (see make_opts), got %s", Py_TYPE(o)->tp_name);
+      throw Failed();
+    }
     if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) throw Failed();
-    if (view.len < (Py_ssize_t)sizeof(uint32_t)) {
+    if (view.len < (Py_ssize_t)sizeof(ersd_opts)) {
       PyBuffer_Release(&view);
-      PyErr_SetString(PyExc_TypeError, "opts must be made by make_opts");
+      PyErr_Format(PyExc_TypeError, "opts has %d bytes, the library's options %d", (int)view.len, (int)sizeof(ersd_opts));
       throw Failed();
     }
     ptr = (const ersd_opts*)view.buf;
@@ -197,12 +206,12 @@ PyObject* guarded(Py_ssize_t n, F&& body) {
 // race_sample(logits, seeds, T, out_tok, opts, stream, V)
 PyObject* race_sample(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return guarded<7>(n, [&]() {
+    const Options o(a[4]);
     tensor(a[0], at::ScalarType::Undefined, "logits");
     const void* seeds = tensor(a[1], at::kLong, "seeds").data_ptr();
     int32_t* out = (int32_t*)tensor(a[3], at::kInt, "out_tok").data_ptr();
     Logits l = logits(a[0], a[6], "logits");
     logits_code(l);
-    const Options o(a[4]);
     const float T = number(a[2]);
     void* st = stream_of(a[5]);
     return status_of([&] { return f_race_sample(l.data, l.code, (const uint64_t*)seeds, l.B, l.rows, l.V, T, out, o.ptr, st); });
@@ -213,13 +222,13 @@ PyObject* race_sample(PyObject*, PyObject* const* a, Py_ssize_t n) {
 template <typename Fn>
 PyObject* verify_with(PyObject* const* a, Py_ssize_t n, Fn fn) {
   return guarded<9>(n, [&]() {
+    const Options o(a[6]);
     Logits l = logits(a[0], a[8], "target_logits");
     const void* draft = optional_tensor(a[1], l.type, "draft_logits");
     const void* seeds = tensor(a[2], at::kLong, "seeds").data_ptr();
     int32_t* tok = (int32_t*)tensor(a[4], at::kInt, "out_tokens").data_ptr();
     int32_t* acc = (int32_t*)tensor(a[5], at::kInt, "out_accept_len").data_ptr();
     logits_code(l);
-    const Options o(a[6]);
     const float T = number(a[3]);
     void* st = stream_of(a[7]);
     return status_of([&] { return fn(l.data, draft, l.code, (const uint64_t*)seeds, l.B, l.rows - 1, l.V, T, tok, acc, o.ptr, st); });
@@ -231,13 +240,13 @@ PyObject* verify_noalloc(PyObject*, PyObject* const* a, Py_ssize_t n) { return v
 // verify_tokens(target, draft_tokens, seeds, T, out_tokens, out_accept_len, opts, stream, V)
 PyObject* verify_tokens(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return guarded<9>(n, [&]() {
+    const Options o(a[6]);
     Logits l = logits(a[0], a[8], "target_logits");
     const void* given = optional_tensor(a[1], at::kInt, "draft_tokens");
     const void* seeds = tensor(a[2], at::kLong, "seeds").data_ptr();
     int32_t* tok = (int32_t*)tensor(a[4], at::kInt, "out_tokens").data_ptr();
     int32_t* acc = (int32_t*)tensor(a[5], at::kInt, "out_accept_len").data_ptr();
     logits_code(l);
-    const Options o(a[6]);
     const float T = number(a[3]);
     void* st = stream_of(a[7]);
     return status_of([&] {
@@ -249,6 +258,7 @@ PyObject* verify_tokens(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // verify_tree(target, draft, parent, seeds, T, out_tokens, out_accept_len, opts, stream, V)
 PyObject* verify_tree(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return guarded<10>(n, [&]() {
+    const Options o(a[7]);
     Logits l = logits(a[0], a[9], "target_logits");
     const void* draft = optional_tensor(a[1], l.type, "draft_logits");
     const void* seeds = tensor(a[3], at::kLong, "seeds").data_ptr();
@@ -256,7 +266,6 @@ PyObject* verify_tree(PyObject*, PyObject* const* a, Py_ssize_t n) {
     int32_t* acc = (int32_t*)tensor(a[6], at::kInt, "out_accept_len").data_ptr();
     const std::vector<int32_t> parent = parents(a[2], l.rows);
     logits_code(l);
-    const Options o(a[7]);
     const float T = number(a[4]);
     void* st = stream_of(a[8]);
     return status_of([&] {
@@ -268,6 +277,7 @@ PyObject* verify_tree(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // gsd_verify(target, draft, draft_tokens, seeds, T, out_tokens, out_accept_len, opts, stream, V)
 PyObject* gsd_verify(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return guarded<10>(n, [&]() {
+    const Options o(a[7]);
     Logits l = logits(a[0], a[9], "target_logits");
     const void* draft = optional_tensor(a[1], l.type, "draft_logits");
     const void* given = optional_tensor(a[2], at::kInt, "draft_tokens");
@@ -275,7 +285,6 @@ PyObject* gsd_verify(PyObject*, PyObject* const* a, Py_ssize_t n) {
     int32_t* tok = (int32_t*)tensor(a[5], at::kInt, "out_tokens").data_ptr();
     int32_t* acc = (int32_t*)tensor(a[6], at::kInt, "out_accept_len").data_ptr();
     logits_code(l);
-    const Options o(a[7]);
     const float T = number(a[4]);
     void* st = stream_of(a[8]);
     return status_of([&] {
@@ -287,6 +296,7 @@ PyObject* gsd_verify(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // gsd_verify_tree(target, draft, draft_tokens, parent, seeds, T, out_tokens, out_accept_len, opts, stream, V)
 PyObject* gsd_verify_tree(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return guarded<11>(n, [&]() {
+    const Options o(a[8]);
     Logits l = logits(a[0], a[10], "target_logits");
     const void* draft = optional_tensor(a[1], l.type, "draft_logits");
     const void* given = optional_tensor(a[2], at::kInt, "draft_tokens");
@@ -295,7 +305,6 @@ PyObject* gsd_verify_tree(PyObject*, PyObject* const* a, Py_ssize_t n) {
     int32_t* acc = (int32_t*)tensor(a[7], at::kInt, "out_accept_len").data_ptr();
     const std::vector<int32_t> parent = parents(a[3], l.rows);
     logits_code(l);
-    const Options o(a[8]);
     const float T = number(a[5]);
     void* st = stream_of(a[9]);
     return status_of([&] {
@@ -305,11 +314,19 @@ PyObject* gsd_verify_tree(PyObject*, PyObject* const* a, Py_ssize_t n) {
   });
 }
 
-// use(race_sample, verify, verify_noalloc, verify_tokens, verify_tree, gsd_verify, gsd_verify_tree): the
-// library's functions, as addresses
+// use(race_sample, verify, verify_noalloc, verify_tokens, verify_tree, gsd_verify, gsd_verify_tree, opts): the
+// library's functions, as addresses, and the type of the options structure
 PyObject* use(PyObject*, PyObject* args) {
   unsigned long long f[7];
-  if (!PyArg_ParseTuple(args, "KKKKKKK", &f[0], &f[1], &f[2], &f[3], &f[4], &f[5], &f[6])) return nullptr;
+  PyObject* type;
+  if (!PyArg_ParseTuple(args, "KKKKKKKO", &f[0], &f[1], &f[2], &f[3], &f[4], &f[5], &f[6], &type)) return nullptr;
+  if (!PyType_Check(type)) {
+    PyErr_SetString(PyExc_TypeError, "the type of the options structure is wanted");
+    return nullptr;
+  }
+  Py_INCREF(type);
+  Py_XDECREF(options_type);
+  options_type = type;
   f_race_sample = (decltype(f_race_sample))(uintptr_t)f[0];
   f_verify = (decltype(f_verify))(uintptr_t)f[1];
   f_verify_noalloc = (decltype(f_verify_noalloc))(uintptr_t)f[2];

@@ -144,3 +144,30 @@ def test_missing_library_fails_loudly(monkeypatch):
     monkeypatch.setattr(binding, "LIB_PATH", "/nonexistent/libersd.so")
     with pytest.raises(RuntimeError, match="no CPU fallback"):
         binding.lib()
+
+
+def test_binding_takes_no_other_object_as_options(L):
+    """The library copies as many bytes as the structure says it has: anything but an ErsdOpts, however
+    long its buffer, is refused before a tensor is looked at."""
+    import torch
+    from paper_2504_15475_b200 import binding
+    t = torch.zeros(1, 1, 8)
+    i = torch.zeros(1, 1, dtype=torch.int32)
+
+    class Short(C.Structure):
+        _fields_ = [("struct_size", C.c_uint32)]
+
+    calls = [lambda o: binding.ersd_race_sample(t, i, 1.0, i, o),
+             lambda o: binding.ersd_verify(t, None, i, 1.0, i, i, o),
+             lambda o: binding.ersd_verify_noalloc(t, None, i, 1.0, i, i, o),
+             lambda o: binding.ersd_verify_tokens(t, None, i, 1.0, i, i, o),
+             lambda o: binding.ersd_verify_tree(t, None, [-1], i, 1.0, i, i, o),
+             lambda o: binding.ersd_gsd_verify(t, None, None, i, 1.0, i, i, o),
+             lambda o: binding.ersd_gsd_verify_tree(t, None, None, [-1], i, 1.0, i, i, o)]
+    for call in calls:
+        for bad in (b"\0" * 4, bytearray(4096), Short(4), (C.c_uint8 * 4096)(), 7):
+            with pytest.raises(TypeError, match="opts must be"):
+                call(bad)
+        for good in (None, binding.make_opts(), type("Mine", (binding.ErsdOpts,), {})()):
+            with pytest.raises(ValueError, match="must be a CUDA tensor"):
+                call(good)
