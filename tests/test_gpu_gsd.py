@@ -270,3 +270,100 @@ def test_long_drafts_that_end_in_exact_races(ersd):
         assert (ws == 0).all(), rep
         assert (acc.cpu().numpy()[ok] == ref["accept_len"][ok]).all()
         assert (out.cpu().numpy()[ok] == ref["tokens"][ok]).all()
+
+
+@pytest.mark.parametrize("T", [1.0, 0.25])
+def test_tokens_whose_probability_is_nothing_in_double_precision(ersd, T):
+    """Given tokens with log2 probabilities from -8 down past the end of double precision's range (2^-1075)
+    and at -inf, under either law, in every combination: ratios of 0, of infinity, 0/0 and ordinary ones.
+    (Between -1080 and -1020, where a probability loses its digits, two exponentials may differ.)"""
+    grid = [float("-inf"), -3000, -1200, -1160, -1140, -1100, -1010, -950, -905, -895, -500, -60, -8]
+    B, V = len(grid) ** 2, 500
+    g = torch.Generator().manual_seed(10)
+    drf = torch.randn(B, 1, V, generator=g)
+    tgt = torch.randn(B, 2, V, generator=g)
+    x = torch.randint(0, V, (B,), generator=g)
+    n = torch.arange(B)
+    for rows, which in ((tgt, n // len(grid)), (drf, n % len(grid))):
+        rest = rows[:, 0].double() / T
+        rest[n, x] = float("-inf")
+        lp = torch.tensor(grid, dtype=torch.float64)[which] * np.log(2.0)
+        rows[n, 0, x] = ((torch.logsumexp(rest, -1) + lp) * T).float()
+    tok = x.view(B, 1).to(torch.int32)
+    seeds = wl.make_seeds(23, 0, B)
+    out = torch.full((B, 2), -9, dtype=torch.int32, device="cuda")
+    acc = torch.full((B,), -9, dtype=torch.int32, device="cuda")
+    ersd.ersd_gsd_verify(tgt.cuda(), drf.cuda(), tok.cuda(), seeds.cuda(), T, out, acc)
+    torch.cuda.synchronize()
+    ref = oracle.gsd_verify(tgt.numpy(), drf.numpy(), tok.numpy(), wl.seeds_as_u64(seeds), T=T)
+    ok = ~ambiguous(ref)
+    assert ok.sum() >= B - 1 and len(grid) < ref["accept_len"].sum() < B - len(grid)
+    assert (acc.cpu().numpy()[ok] == ref["accept_len"][ok]).all()
+    assert (out.cpu().numpy()[ok] == ref["tokens"][ok]).all()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("V", [7, 40001, 128256])
+def test_rows_that_are_no_law(ersd, V, dtype):
+    """A logit of +inf (the drafted token's or another one's), or none above -inf, in the target row, the
+    draft row or the last row: nothing is accepted there and nothing emitted; and the masked token of an
+    ordinary row."""
+    B, k = 12, 3
+    w = wl.Workload("gsdlaw", B=B, k=k, V=V, dtype=dtype, sigma=0.3, T=0.9, config_id=53)
+    inp = wl.make_inputs(w)
+    tgt, drf, inf = inp["target"], inp["draft"], float("inf")
+    tok = draft_tokens(ersd, drf.cuda(), inp["seeds"].cuda(), inp["T"])[..., 0].contiguous()
+    x = tok.cpu().long()
+    tgt[0, 0, x[0, 0]] = inf
+    tgt[1, 1, V // 2] = inf
+    drf[2, 0, x[2, 0]] = inf
+    drf[3, 2, V - 1] = inf
+    tgt[4, k, 0] = inf
+    tgt[5, k] = -inf
+    tgt[6, 0] = -inf
+    drf[7, 0] = -inf
+    tgt[8, 0, x[8, 0]] = -inf
+    drf[9, 0, x[9, 0]] = -inf
+    tgt[10, 0, :] = float("nan")
+    tgt[11, 0, 1:] = -inf
+    out = torch.full((B, k + 1), -9, dtype=torch.int32, device="cuda")
+    acc = torch.full((B,), -9, dtype=torch.int32, device="cuda")
+    for rep in range(2):
+        ersd.ersd_gsd_verify(tgt.cuda(), drf.cuda(), tok, inp["seeds"].cuda(), inp["T"], out, acc)
+    torch.cuda.synchronize()
+    ref = oracle.gsd_verify(wl.as_numpy_logits(tgt), wl.as_numpy_logits(drf), tok.cpu().numpy(),
+                            wl.seeds_as_u64(inp["seeds"]), T=inp["T"])
+    ok = ~ambiguous(ref)
+    assert ok.sum() >= B - 1
+    assert (acc.cpu().numpy()[ok] == ref["accept_len"][ok]).all()
+    assert (out.cpu().numpy()[ok] == ref["tokens"][ok]).all()
+
+
+def test_masked_and_infinite_logits_take_no_second_reading(ersd):
+    """A drafted token that the target's mask rules out, and a row with a logit of +inf, are decided by the
+    sums that every call takes.  (Read again in double precision by one block such a call took 153 and 530 us,
+    an ordinary one 14: a factor of three leaves room for a disturbed clock.)"""
+    w = wl.scaled(wl.CONFIGS["c5"], B=1)
+    inp = wl.make_inputs(w, device="cuda")
+    tgt, drf, seeds = inp["target"], inp["draft"], inp["seeds"]
+    tok = draft_tokens(ersd, drf, seeds, 1.0)[..., 0].contiguous()
+    masked, infinite = tgt.clone(), tgt.clone()
+    masked[0, 0, tok[0, 0].item()] = float("-inf")
+    infinite[0, 0, 5] = float("inf")
+    out = torch.empty(1, w.k + 1, dtype=torch.int32, device="cuda")
+    acc = torch.empty(1, dtype=torch.int32, device="cuda")
+
+    def us(t):
+        best = float("inf")
+        for rep in range(12):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for q in range(20):
+                ersd.ersd_gsd_verify(t, drf, tok, seeds, 1.0, out, acc)
+            e1.record()
+            e1.synchronize()
+            best = min(best, e0.elapsed_time(e1) * 50.0)
+        return best
+
+    plain = us(tgt)
+    assert us(masked) < 3.0 * plain and us(infinite) < 3.0 * plain
