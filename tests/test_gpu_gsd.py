@@ -367,3 +367,31 @@ def test_masked_and_infinite_logits_take_no_second_reading(ersd):
 
     plain = us(tgt)
     assert us(masked) < 3.0 * plain and us(infinite) < 3.0 * plain
+
+
+@pytest.mark.parametrize("T", [0.05, 0.2])
+@pytest.mark.parametrize("V", [3001, 40000])
+def test_tokens_drafted_at_another_temperature(ersd, V, T):
+    """Given tokens that the laws at a low temperature would hardly draw: rejected, and then the residual
+    hangs on the last digits of one token's two probabilities, so the last race is run in double precision.
+    A difference of less than 1e-9 of them is left out: both are known to a few 2^-53, so its own error passes
+    1e-6, a tenth of the window inside which two arrivals may come either way."""
+    B, k = 64, 2
+    w = wl.Workload("gsdcold", B=B, k=k, V=V, dtype="bf16", sigma=0.3, T=T, config_id=54)
+    inp = wl.make_inputs(w)
+    tok = draft_tokens(ersd, inp["draft"].cuda(), inp["seeds"].cuda(), 1.0)[..., 0].contiguous()
+    out = torch.full((B, k + 1), -9, dtype=torch.int32, device="cuda")
+    acc = torch.full((B,), -9, dtype=torch.int32, device="cuda")
+    ersd.ersd_gsd_verify(inp["target"].cuda(), inp["draft"].cuda(), tok, inp["seeds"].cuda(), T, out, acc)
+    torch.cuda.synchronize()
+    ref = oracle.gsd_verify(wl.as_numpy_logits(inp["target"]), wl.as_numpy_logits(inp["draft"]), tok.cpu().numpy(),
+                            wl.seeds_as_u64(inp["seeds"]), T=T)
+    n, L = np.arange(B), np.minimum(ref["accept_len"], k - 1)
+    p = torch.softmax(inp["target"][n, L].double() / T, -1)
+    q = torch.softmax(inp["draft"][n, L].double() / T, -1)
+    either = torch.maximum(p, q)
+    close = ((either > 1e-3) & ((p - q).abs() < 1e-9 * either)).any(-1).numpy()
+    ok = ~ambiguous(ref) & ~close
+    assert ok.sum() >= B // 2 and (ref["accept_len"] == 0).sum() >= B // 4
+    assert (acc.cpu().numpy()[ok] == ref["accept_len"][ok]).all()
+    assert (out.cpu().numpy()[ok] == ref["tokens"][ok]).all()
