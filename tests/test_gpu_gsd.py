@@ -395,3 +395,26 @@ def test_tokens_drafted_at_another_temperature(ersd, V, T):
     assert ok.sum() >= B // 2 and (ref["accept_len"] == 0).sum() >= B // 4
     assert (acc.cpu().numpy()[ok] == ref["accept_len"][ok]).all()
     assert (out.cpu().numpy()[ok] == ref["tokens"][ok]).all()
+
+
+@pytest.mark.parametrize("k,V", [(31, 900), (32, 1025), (127, 1025), (128, 3000), (200, 1000), (255, 40), (60, 40000)])
+def test_long_drafts_of_short_rows(ersd, k, V):
+    """Rows of one slice and of several, more rows than a block's warps or lanes take at a time, runs of
+    accepted tokens that end in the middle of 32, at their end and at the last row."""
+    B = 6
+    w = wl.Workload("gsdrun", B=B, k=k, V=V, dtype="f32", sigma=0.02, T=1.0, config_id=55)
+    inp = wl.make_inputs(w)
+    tok = draft_tokens(ersd, inp["draft"].cuda(), inp["seeds"].cuda(), inp["T"])[..., 0].contiguous()
+    inp["draft"][0] = inp["target"][0, :k]                      # (all accepted)
+    inp["target"][1, 31 % k] = float("-inf")
+    inp["target"][2, min(32, k - 1)] = float("-inf")
+    out = torch.full((B, k + 1), -9, dtype=torch.int32, device="cuda")
+    acc = torch.full((B,), -9, dtype=torch.int32, device="cuda")
+    ersd.ersd_gsd_verify(inp["target"].cuda(), inp["draft"].cuda(), tok, inp["seeds"].cuda(), inp["T"], out, acc)
+    torch.cuda.synchronize()
+    ref = oracle.gsd_verify(wl.as_numpy_logits(inp["target"]), wl.as_numpy_logits(inp["draft"]), tok.cpu().numpy(),
+                            wl.seeds_as_u64(inp["seeds"]), T=inp["T"])
+    ok = ~ambiguous(ref)
+    assert ok.sum() >= B - 1 and ref["accept_len"][0] == k
+    assert (acc.cpu().numpy()[ok] == ref["accept_len"][ok]).all()
+    assert (out.cpu().numpy()[ok] == ref["tokens"][ok]).all()
