@@ -115,7 +115,8 @@ typedef struct ersd_opts {
                               (one thread-block cluster per position; one kernel for races of one arrival, one
                               for races of up to 32: top_c > 1, trees with branching;
                               ERSD_EUNSUPPORTED where neither applies: a race of more than 32 arrivals,
-                              rows not 16-byte aligned (the library's own choice takes those too), B or R > 65535, more than 32 rows per sequence
+                              rows not 16-byte aligned (the library's own choice takes those too), B or
+                              R > 65535, more than 32 rows per sequence
                               in ersd_verify and its variants, near_tie_count given, or a vocabulary too
                               long for eight blocks to stage in shared memory: beyond about 320 k entries
                               in bf16, 160 k in fp32, halved when draft rows are raced along, less the
