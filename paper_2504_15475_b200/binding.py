@@ -107,8 +107,12 @@ def native():
         try:
             from . import _ersd_call
         except ImportError as e:
-            raise RuntimeError("_ersd_call.so not found next to %s: run `python -m paper_2504_15475_b200.build` (%s)"
-                               % (__file__, e)) from None
+            raise RuntimeError("_ersd_call.so next to %s is missing or cannot be loaded: run `python -m "
+                               "paper_2504_15475_b200.build` (%s)" % (__file__, e)) from None
+        built_for = getattr(_ersd_call, "torch_version", "another version")
+        if built_for != str(torch.__version__):
+            raise RuntimeError("_ersd_call.so was built against torch %s, this is %s: run `python -m "
+                               "paper_2504_15475_b200.build`" % (built_for, torch.__version__))
         _ersd_call.use(*[C.cast(f, C.c_void_p).value for f in (
             L.ersd_race_sample, L.ersd_verify, L.ersd_verify_noalloc, L.ersd_verify_tokens, L.ersd_verify_tree,
             L.ersd_gsd_verify, L.ersd_gsd_verify_tree)], ErsdOpts)

@@ -31,6 +31,7 @@ def call_command(out: str):
     cuda = os.path.dirname(os.path.dirname(os.path.realpath(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc")))
     return ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
             "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+            '-DERSD_TORCH_VERSION="%s"' % torch.__version__,
             "-I", os.path.join(ROOT, "include"), "-I", os.path.join(root, "include"),
             "-I", os.path.join(root, "include", "torch", "csrc", "api", "include"),
             "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include"), CALL_SRC, "-o", out,
@@ -41,11 +42,20 @@ def _fresh(lib: str, deps) -> bool:
     return os.path.exists(lib) and all(os.path.getmtime(lib) >= os.path.getmtime(d) for d in deps)
 
 
+def _call_fresh() -> bool:
+    """Whether the extension module is newer than its sources and built against the installed torch."""
+    import torch
+    if not _fresh(CALL_LIB, [CALL_SRC, os.path.join(ROOT, "include", "ersd.h")]):
+        return False
+    with open(CALL_LIB, "rb") as f:
+        return b"\0" + str(torch.__version__).encode() + b"\0" in f.read()
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     jobs = []
     if force or not _fresh(LIB, DEPS):
         jobs.append((LIB, lambda out: nvcc_command(out, ("-Xptxas", "-v") if verbose else ())))
-    if force or not _fresh(CALL_LIB, [CALL_SRC, os.path.join(ROOT, "include", "ersd.h")]):
+    if force or not _call_fresh():
         jobs.append((CALL_LIB, call_command))
     running = []
     for lib, command in jobs:

@@ -344,4 +344,9 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_ersd_call", nullptr, -1, methods,
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__ersd_call() { return PyModule_Create(&module); }
+// (torch_version: the torch this was built against, whose tensors alone it can take apart)
+PyMODINIT_FUNC PyInit__ersd_call() {
+  PyObject* m = PyModule_Create(&module);
+  if (m && PyModule_AddStringConstant(m, "torch_version", ERSD_TORCH_VERSION) != 0) Py_CLEAR(m);
+  return m;
+}

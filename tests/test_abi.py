@@ -171,3 +171,16 @@ def test_binding_takes_no_other_object_as_options(L):
         for good in (None, binding.make_opts(), type("Mine", (binding.ErsdOpts,), {})()):
             with pytest.raises(ValueError, match="must be a CUDA tensor"):
                 call(good)
+
+
+def test_extension_module_of_another_torch(L, monkeypatch):
+    """Says so instead of failing somewhere in a call, and is built anew."""
+    import torch
+    from paper_2504_15475_b200 import binding
+    assert ersd_build._call_fresh()
+    assert binding.native().torch_version == str(torch.__version__)
+    monkeypatch.setattr(binding, "_native", None)
+    monkeypatch.setattr(torch, "__version__", "1.0.0")
+    assert not ersd_build._call_fresh()
+    with pytest.raises(RuntimeError, match="built against torch"):
+        binding.native()
