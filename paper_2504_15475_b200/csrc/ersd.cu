@@ -402,33 +402,54 @@ static RaceKernel race_kernel(bool bf16, bool aligned, bool many, int threads) {
   return aligned ? race_kernel_of<ERSD_F32, true>(many, threads) : race_kernel_of<ERSD_F32, false>(many, threads);
 }
 
-// Four resident blocks per SM need about 180 KB of shared memory: ask for the largest carveout
-// (a hint to the driver; set once per device and kernel).
-static int prefer_shared_memory() {
+// What a kernel needs before its first launch on a device: its dynamic shared memory allowed, and
+//   carveout: the largest shared-memory carveout asked for (a hint to the driver: four resident blocks of
+//             the streaming kernel need about 180 KB);
+//   cluster:  the opt-in for clusters of 16 blocks; *limit = the largest cluster (a power of two) that it
+//             can be launched in: 16 where that is granted and such a cluster fits, else 8.
+// Done when a call first wants the kernel: the attributes load its code, and asking for all the cluster
+// builds' at once made a process's first call take 35 ms (10 when there were eight of them).
+struct KernelState {
+  const void* kernel;
+  uint64_t ready, sixteen;  // bits: devices
+};
+static int prepare_kernel(const void* kernel, size_t smem, bool carveout, bool cluster, int* limit) {
   static std::mutex m;
-  static bool done[64];
+  static KernelState known[64];  // (as many as there are builds)
+  static int count;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return cuda_fail(e);
   if (dev < 0 || dev >= 64) return ERSD_EUNSUPPORTED;
+  const uint64_t bit = (uint64_t)1 << dev;
   std::lock_guard<std::mutex> lock(m);
-  if (!done[dev]) {
-    e = cudaSuccess;
-    auto prefer = [&](const void* kernel, size_t smem) {
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    };
-    for (int bf16 = 0; bf16 < 2; ++bf16)
-      for (int aligned = 0; aligned < 2; ++aligned)
-        for (int many = 0; many < 2; ++many)
-          for (int threads = 128; threads <= 256; threads += 128) {
-            const RaceKernel k = race_kernel(bf16 != 0, aligned != 0, many != 0, threads);
-            prefer((const void*)k.kernel, k.smem);
-          }
-    if (e != cudaSuccess) return cuda_fail(e);
-    done[dev] = true;
+  int at = 0;
+  while (at < count && known[at].kernel != kernel) ++at;
+  KernelState fresh = {kernel, 0, 0};
+  KernelState& k = at < 64 ? known[at] : fresh;
+  if (at == count && at < 64) {
+    k = fresh;
+    ++count;
   }
+  if (!(k.ready & bit)) {
+    if (carveout) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess && smem) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return cuda_fail(e);
+    if (cluster) {
+      int n = 0;
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e == cudaSuccess) {
+        Launch l(dim3(16, 1, 1), b256::kThreads, smem, nullptr, 16);
+        l.cfg.attrs = &l.at[1];  // (the cluster's size alone)
+        l.cfg.numAttrs = 1;
+        e = cudaOccupancyMaxActiveClusters(&n, kernel, &l.cfg);
+      }
+      if (e == cudaSuccess && n >= 1) k.sixteen |= bit;
+      (void)cudaGetLastError();  // a refused opt-in only means clusters of eight
+    }
+    k.ready |= bit;
+  }
+  if (limit) *limit = (k.sixteen & bit) ? 16 : 8;
   return ERSD_OK;
 }
 
@@ -445,11 +466,11 @@ static int launch(const Params& p, const TreeDesc& tree, int dt, int cmax, cudaS
   // is the chunk-major order the kernel counts on, and the kernel needs no division to decode
   if (p.rows > 65535 || p.S > 65535) return ERSD_EUNSUPPORTED;
   const dim3 grid((unsigned)p.B, (unsigned)p.rows, (unsigned)p.S);
-  const int pst = prefer_shared_memory();
+  const RaceKernel k = race_kernel(dt == ERSD_BF16, p.aligned_t && p.aligned_d, many, p.threads);
+  const int pst = prepare_kernel((const void*)k.kernel, k.smem, true, false, nullptr);
   if (pst != ERSD_OK) return pst;
   snprintf(g_last_launch, sizeof g_last_launch, "ersd_race_kernel<%s>%s: %d threads x (%d, %d, %d) blocks, %d chunk(s) per row",
            dt == ERSD_BF16 ? "bf16" : "f32", many ? " (pooled thresholds)" : "", p.threads, p.B, p.rows, p.S, p.S);
-  const RaceKernel k = race_kernel(dt == ERSD_BF16, p.aligned_t && p.aligned_d, many, p.threads);
   Launch l(grid, (unsigned)p.threads, k.smem, st);
   const cudaError_t e = cudaLaunchKernelEx(&l.cfg, k.kernel, p, tree);
   return e == cudaSuccess ? ERSD_OK : cuda_fail(e);
@@ -491,65 +512,19 @@ static int cluster_max_tiles(int dt, int roles, int cmax, bool aligned) {
   return (int)((kClusterSmemBytes - lists) / (per_tile * (size_t)roles));
 }
 
-// Largest cluster (a power of two) the device takes for the cluster kernels: 16 where the opt-in
-// for non-portable sizes is granted and such a cluster fits, else 8.  Asked once per device.
-static int cluster_limit(int* out) {
-  static std::mutex m;
-  static int limit[64];
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return cuda_fail(e);
-  if (dev < 0 || dev >= 64) return ERSD_EUNSUPPORTED;
-  std::lock_guard<std::mutex> lock(m);
-  if (!limit[dev]) {
-    constexpr int kKernels = 32, kSmall = 8;  // (the last kSmall: 128-thread blocks, never in clusters)
-    const void* kernels[kKernels + kSmall];
-    int count = 0, small = kKernels;
-    auto add = [&](auto dt, auto nr, auto al) {
-      kernels[count++] = (const void*)b256::ersd_cluster_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value, true>;
-      kernels[count++] = (const void*)b256::ersd_cluster_top_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value, true>;
-      kernels[count++] = (const void*)b256::ersd_cluster_top_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value, false>;
-      kernels[count++] = (const void*)b256::ersd_cluster_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value, false>;
-      kernels[small++] = (const void*)b128::ersd_cluster_kernel<decltype(dt)::value, decltype(nr)::value, decltype(al)::value, true>;
-    };
-    auto both = [&](auto dt, auto nr) {
-      add(dt, nr, std::true_type());
-      add(dt, nr, std::false_type());
-    };
-    both(std::integral_constant<int, ERSD_BF16>(), std::integral_constant<int, 1>());
-    both(std::integral_constant<int, ERSD_BF16>(), std::integral_constant<int, 2>());
-    both(std::integral_constant<int, ERSD_F32>(), std::integral_constant<int, 1>());
-    both(std::integral_constant<int, ERSD_F32>(), std::integral_constant<int, 2>());
-    int lim = 16;
-    for (int q = 0; q < kKernels + kSmall; ++q) {
-      e = cudaFuncSetAttribute(kernels[q], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmemBytes);
-      if (e != cudaSuccess) return cuda_fail(e);
-    }
-    for (int q = 0; q < kKernels && lim == 16; ++q) {
-      e = cudaFuncSetAttribute(kernels[q], cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      int n = 0;
-      if (e == cudaSuccess) {
-        cudaLaunchConfig_t cfg;
-        memset(&cfg, 0, sizeof cfg);
-        cfg.gridDim = dim3(16, 1, 1);
-        cfg.blockDim = dim3(b256::kThreads, 1, 1);
-        cfg.dynamicSmemBytes = kClusterSmemBytes;
-        cudaLaunchAttribute at;
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = 16;
-        at.val.clusterDim.y = 1;
-        at.val.clusterDim.z = 1;
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
-        e = cudaOccupancyMaxActiveClusters(&n, kernels[q], &cfg);
-      }
-      if (e != cudaSuccess || n < 1) lim = 8;
-    }
-    (void)cudaGetLastError();  // a refused opt-in only means clusters of eight
-    limit[dev] = lim;
+// The build of the cluster kernels for rows of type DT, aligned (AL) or not, `roles` of them raced together.
+template <int DT, bool AL>
+static const void* cluster_kernel(int cmax, int roles, bool staged, bool small) {
+  if (cmax > 1) {
+    if (staged) return roles == 2 ? (const void*)b256::ersd_cluster_top_kernel<DT, 2, AL, true> : (const void*)b256::ersd_cluster_top_kernel<DT, 1, AL, true>;
+    return roles == 2 ? (const void*)b256::ersd_cluster_top_kernel<DT, 2, AL, false> : (const void*)b256::ersd_cluster_top_kernel<DT, 1, AL, false>;
   }
-  *out = limit[dev];
-  return ERSD_OK;
+  if (small) {
+    if (staged) return roles == 2 ? (const void*)b128::ersd_cluster_kernel<DT, 2, AL, true> : (const void*)b128::ersd_cluster_kernel<DT, 1, AL, true>;
+    return roles == 2 ? (const void*)b128::ersd_cluster_kernel<DT, 2, AL, false> : (const void*)b128::ersd_cluster_kernel<DT, 1, AL, false>;
+  }
+  if (staged) return roles == 2 ? (const void*)b256::ersd_cluster_kernel<DT, 2, AL, true> : (const void*)b256::ersd_cluster_kernel<DT, 1, AL, true>;
+  return roles == 2 ? (const void*)b256::ersd_cluster_kernel<DT, 2, AL, false> : (const void*)b256::ersd_cluster_kernel<DT, 1, AL, false>;
 }
 
 // Whether a call can take a cluster kernel at all; cmax: most arrivals any of its races wants.
@@ -603,10 +578,8 @@ static int unstaged_size(const Params& p, int dt, int roles, int cmax, int lim) 
 // kClusterGroups tiles (shortest path through one position).  Once such clusters would make more
 // than two blocks per SM: blocks of about twice as many tiles (measured at V = 128256: clusters
 // of 8 beat clusters of 16 from about 20 positions on, clusters of 4 never beat clusters of 8).
-static int cluster_size(const ersd_opts& o, const Params& p, int dt, int cmax, bool staged, int* out) {
-  int lim = 8;
-  const int ls = cluster_limit(&lim);
-  if (ls != ERSD_OK) return ls;
+// lim: the largest cluster that the kernel can be launched in.
+static int cluster_size(const ersd_opts& o, const Params& p, int dt, int cmax, bool staged, int lim, int* out) {
   const int ntiles = (p.V + b256::kTile - 1) / b256::kTile;
   const int roles = (p.mode == kVerify && p.draft) ? 2 : 1;
   const int max_tiles = cluster_max_tiles(dt, roles, cmax, p.aligned_t && p.aligned_d);
@@ -646,7 +619,9 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   int roles = (p.mode == kVerify && p.draft) ? 2 : 1;
   int CL = 1;
   const bool staged = cluster_staged(p, DT, roles, cmax);
-  const int ls = cluster_size(o, p, DT, cmax, staged, &CL);
+  int lim = 8;
+  int ls = prepare_kernel(cluster_kernel<DT, AL>(cmax, roles, staged, false), kClusterSmemBytes, false, true, &lim);
+  if (ls == ERSD_OK) ls = cluster_size(o, p, DT, cmax, staged, lim, &CL);
   if (ls != ERSD_OK) return ls;
   const int ntiles = (p.V + b256::kTile - 1) / b256::kTile;
   // Trees of few positions: a cluster per ROW (a node's draft row and its target row side by side
@@ -664,6 +639,10 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
       split = true;
     }
     if (split) {
+      ls = prepare_kernel(cluster_kernel<DT, AL>(cmax, 1, staged, false), kClusterSmemBytes, false, true, &lim);
+      if (ls != ERSD_OK) return ls;
+    }
+    if (split && CL <= lim) {
       p.top_split = 1 + with_children;
       jobs = p.rows + with_children;
       roles = 1;
@@ -676,7 +655,6 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   // instead of 10.4 us); not where the staged rows would leave fewer than five such blocks to an SM.
   // Unstaged rows leave that room up to 16384 logits and beyond; longer ones keep 256 threads busy
   // (800 positions of 15048 logits: 25.8 us with 128 threads, 27.0 with 256; 1200 of 32000 57.1 and 51.4).
-  
   const int G128 = (p.V + b128::kTile - 1) / b128::kTile;
   const bool small = cmax == 1 && CL == 1 && ((int64_t)p.B * p.rows > 4 * sm_count() || G128 == 1) &&
                      (staged ? b128::cluster_role_bytes<DT>(G128, AL) * (size_t)roles <= 41 * 1024 : G128 <= 16);
@@ -694,19 +672,13 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   snprintf(g_last_launch, sizeof g_last_launch, "%s<%s, %d row(s) per cluster>: %d clusters of %d x %d threads, %d positions%s",
            cmax > 1 ? "ersd_cluster_top_kernel" : "ersd_cluster_kernel", DT == ERSD_BF16 ? "bf16" : "f32", roles,
            p.B * jobs, CL, threads, p.B * p.rows, staged ? "" : " (unstaged)");
-  cudaError_t e;
-  if (cmax > 1) {
-    auto kernel = roles == 2 ? b256::ersd_cluster_top_kernel<DT, 2, AL, true> : b256::ersd_cluster_top_kernel<DT, 1, AL, true>;
-    if (!staged) kernel = roles == 2 ? b256::ersd_cluster_top_kernel<DT, 2, AL, false> : b256::ersd_cluster_top_kernel<DT, 1, AL, false>;
-    e = cudaLaunchKernelEx(&l.cfg, kernel, p, tree);
-  } else {
-    void (*kernel)(Params);
-    if (staged && small) kernel = roles == 2 ? b128::ersd_cluster_kernel<DT, 2, AL, true> : b128::ersd_cluster_kernel<DT, 1, AL, true>;
-    else if (staged) kernel = roles == 2 ? b256::ersd_cluster_kernel<DT, 2, AL, true> : b256::ersd_cluster_kernel<DT, 1, AL, true>;
-    else if (small) kernel = roles == 2 ? b128::ersd_cluster_kernel<DT, 2, AL, false> : b128::ersd_cluster_kernel<DT, 1, AL, false>;
-    else kernel = roles == 2 ? b256::ersd_cluster_kernel<DT, 2, AL, false> : b256::ersd_cluster_kernel<DT, 1, AL, false>;
-    e = cudaLaunchKernelEx(&l.cfg, kernel, p);
+  const void* kernel = cluster_kernel<DT, AL>(cmax, roles, staged, small);
+  if (small) {  // (the other builds are prepared by now)
+    ls = prepare_kernel(kernel, staged ? kClusterSmemBytes : 0, false, false, nullptr);
+    if (ls != ERSD_OK) return ls;
   }
+  void* args[] = {&p, const_cast<TreeDesc*>(&tree)};  // (the kernel for one arrival has the first alone)
+  const cudaError_t e = cudaLaunchKernelExC(&l.cfg, kernel, args);
   return e == cudaSuccess ? ERSD_OK : cuda_fail(e);
 }
 
