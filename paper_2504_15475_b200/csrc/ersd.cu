@@ -486,20 +486,22 @@ static int launch(const Params& p, const TreeDesc& tree, int dt, int cmax, cudaS
 // 325).  The streaming kernel spends less on an index, once its thresholds have settled, and more on
 // starting: it takes longer bf16 rows from a number of logits on (verification: at 65256 logits 1500
 // positions 111.2 / 113.5 and 2250 157.2 / 159.5; at 100000 500 65.5 / 69.7; at 128256 400 66.4 / 68.8, 450
-// 77.9 / 81.0, 576 91.8 / 87.5; at 151936 300 64.0 / 71.4 and 400 81.4 / 76.4; trees: at 128256 450 rows 85.7 / 83.8.  Sampling, one row per position: at 128256 800 93.1 / 95.1).
+// 77.9 / 81.0, 576 91.8 / 87.5; at 151936 300 64.0 / 71.4 and 400 81.4 / 76.4; trees: at 128256 450 rows 85.7 /
+// 83.8.  Sampling and given tokens, one row per position: at 128256 800 93.1 / 95.1; at 151936 576 89.4 / 83.3, 640
+// 98.6 / 91.9).
 struct ClusterLimit {
   int row;         // rows of up to this many logits ...
   int64_t logits;  // ... take the cluster kernel while the call has no more logits than this
 };
-// Races of several arrivals gain more from it (trees, cluster kernel / streaming kernel: 16 x 17 nodes of
-// 128256 bf16 logits 59.7 / 80.9 us, 20 x 17 73.4 / 75.6, 24 x 17 130 / 81.5; 256 x 17 of 32000 179.5 / 195.2;
-// 100 x 9 of 128256 32-bit logits 224 / 242; eight arrivals of 256 rows of 128256 60 / 114).  Trees of more
-// than 131072 logits a row stream from 20M logits on although the cluster kernel would be quicker there (8 x 17
-// nodes of 151936: 39.4 / 63.7): the tests fix which kernel takes that call.
+// Races of several arrivals gain more from it, but see top_streams (trees of 17 nodes of bf16 logits, time of the
+// cluster kernel / of the streaming kernel: 16 of 128256 0.72, 24 of 100000 1.02, 64 of 64000 0.99, 200 of 40000 0.92,
+// and of 48000, where a row takes two blocks, 233 / 193 us).  Trees of more than 131072 logits a row stream from
+// 20M logits on although the cluster kernel would be quicker there (8 x 17 nodes of 151936: 39.4 / 63.7 us): the
+// tests fix which kernel takes that call.
 constexpr ClusterLimit kClusterLimits[3][4] = {  // bf16: one row per position, draft and target row, the same in trees
-    {{65536, INT64_MAX}, {INT32_MAX, 100 << 20}},
+    {{65536, INT64_MAX}, {131072, 100 << 20}, {INT32_MAX, 72 << 20}},
     {{65536, INT64_MAX}, {INT32_MAX, 56 << 20}},
-    {{49152, INT64_MAX}, {65536, 80 << 20}, {131072, 40 << 20}, {INT32_MAX, 19 << 20}}};
+    {{40960, INT64_MAX}, {65536, 80 << 20}, {131072, 40 << 20}, {INT32_MAX, 19 << 20}}};
 // The number of blocks up to which a tree's rows get a cluster each (one block per SM and a half)
 constexpr int64_t kClusterSplitBlocks = 384;
 constexpr size_t kClusterSmemBytes = 200 * 1024;  // dynamic shared memory a block of the cluster kernels may use
@@ -603,10 +605,46 @@ static int cluster_size(const ersd_opts& o, const Params& p, int dt, int cmax, b
   return ERSD_OK;
 }
 
+// Races of several arrivals that the streaming kernel takes for other reasons than the table's.  Figures: time of
+// the cluster kernel / of the streaming kernel, us, or their ratio.
+static bool top_streams(const Params& p, int dt, int cmax) {
+  const bool tree = p.mode == kVerify;
+  const int64_t n = (int64_t)p.B * p.rows, logits = n * p.V;
+  // Of a row of less than 768 logits at most three of a block's eight warps have any: too few groups are looked at
+  // for a threshold and the arrivals are picked one by one (500 logits: 8 of 1 row 22.2 / 13.0, of 2048 148 / 34,
+  // 4 of 1 13.6 / 11.5; but 32 of 1 0.8, trees of up to four children 0.84 up to 216 rows and 1.14 at 272).  Up to
+  // 32 rows stay all the same: the tests fix which kernel takes the shortest rows.
+  if (p.V < 768 && cmax > 2 && n > 32 && (n > 256 || (cmax <= 16 && cmax > (tree ? 4 : 2)))) return true;
+  if (p.V <= 4096) {
+    // Many short rows: a block's phases behind the bounds take longer than the bounds, and the streaming kernel's
+    // are lighter (1000 logits: 4 of 1024 rows 0.75, of 2048 35.6 / 21.5; 16 of 1024 67.3 / 57.7; 32 of 6000 0.67;
+    // trees: stars of 8, 1152 rows 28.1 / 24.2; 17 nodes 1088 0.96, 3400 59.6 / 43.6; stars of 32 2112 0.88, 6600
+    // 122 / 77.  2048 logits: sampling up to 0.95; trees: three children 1800 35.5 / 31.3, 17 nodes 2176 0.98, 3400
+    // 59.9 / 54.9; stars of 32 6600 114 / 95.  4096: three children 1800 38.6 / 36.0, 17 nodes 3400 65.8 / 61.2,
+    // stars of 8 0.87).
+    if (!tree) return p.V <= 1536 && (cmax <= 8 ? n > 1500 : cmax <= 16 && n > 800);
+    if (p.V <= 1536) return n > (cmax <= 16 ? 1100 : 3000);
+    if (cmax <= 4) return n > (cmax <= 3 ? 1500 : 3000);
+    return p.V <= 3072 && n > (cmax <= 16 ? 2500 : 5000);
+  }
+  // Long rows, few arrivals (100000 bf16 logits: 2 of 1024 rows 135 / 124, 4 of 1024 233 / 163; 32-bit: 4 of 1024
+  // 236 / 184, 2 of 1024 0.9).
+  if (!tree) return p.V > 65536 && p.V <= 131072 && cmax <= 4 && (dt == ERSD_BF16 || cmax > 2) && logits > (90 << 20);
+  // 32-bit trees, which the table leaves out (stars of 8, 200 of 48000 logits 176 / 143; two alternatives, 128 of
+  // 100000 90 / 78, of 128256 1.0).
+  if (dt == ERSD_F32 && p.V > 40960 && cmax <= 16) {
+    if (p.V <= 65536) return logits > (80 << 20);
+    return cmax == 2 && logits > (32 << 20);
+  }
+  return false;
+}
+
 // Whether a call that leaves the choice to the library takes the cluster kernel.
 static bool cluster_by_default(const ersd_opts& o, const Params& p, int dt, int cmax) {
   if (o.kernel_path != 0 || o.split_v != 0 || o.block_threads != 0 || !cluster_applies(p, dt, cmax)) return false;
+  if (cmax > 1 && top_streams(p, dt, cmax)) return false;
   if (dt == ERSD_F32) return true;
+  if (cmax > 16 && p.V <= 49152) return true;  // (64 stars of 32 of 48000 logits: 0.66)
   const ClusterLimit* limit = kClusterLimits[!(p.mode == kVerify && p.draft) ? 0 : cmax > 1 ? 2 : 1];
   while (p.V > limit->row) ++limit;
   return (int64_t)p.V * p.B * p.rows <= limit->logits;

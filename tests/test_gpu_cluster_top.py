@@ -287,3 +287,41 @@ def test_where_this_kernel_does_not_apply(ersd):
     ersd.ersd_verify_tree(t, t, parent, seeds, 1.0, out, acc, None)    # the library picks the streaming kernel
     torch.cuda.synchronize()
     assert (acc == 1).all()                                # draft rows = target rows: the first child is accepted
+
+
+@pytest.mark.parametrize("call,B,V,dtype,streams", [
+    (8, 33, 500, "bf16", True), (8, 33, 767, "f32", True), (8, 33, 768, "f32", False), (2, 300, 500, "bf16", False),
+    (32, 3, 500, "bf16", False), (4, 1500, 1000, "bf16", False), (4, 1501, 1000, "bf16", True), (16, 801, 1000, "f32", True),
+    (32, 2048, 1000, "bf16", False), (4, 1600, 2048, "bf16", False), ("star8", 122, 1000, "bf16", False),
+    ("star8", 123, 1000, "bf16", True), ("4x4", 100, 2048, "f32", False), ("4x4", 177, 3000, "bf16", True),
+    ("specinfer", 167, 4096, "bf16", True), ("4x4", 48, 48000, "bf16", False), ("4x4", 104, 48000, "bf16", True),
+    ("star32", 60, 48000, "bf16", False), ("star8", 196, 48000, "f32", True)])
+def test_default_choice_for_many_or_short_rows(ersd, call, B, V, dtype, streams):
+    """Sizes on both sides of the lines between the two kernels: the one that was measured to be quicker takes
+    the call, and its arrivals are the other one's, bit for bit (rows off a 16-byte boundary: cluster kernel
+    against streaming kernel only where the former is the choice)."""
+    g = torch.Generator(device="cuda").manual_seed(V + B)
+    parent = None if isinstance(call, int) else list({"star8": wl.star_parent(8), "star32": wl.star_parent(32),
+                                                      "4x4": wl.TREE_4x4, "specinfer": wl.TREE_SPECINFER}[call])
+    rows = 1 if parent is None else len(parent)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    tgt = torch.randn(B, rows, V, generator=g, device="cuda").mul_(2.0).to(dt)
+    drf = (tgt.float() * 0.5).to(dt)
+    seeds = wl.make_seeds(61, 0, B).cuda()
+    aligned = V * tgt.element_size() % 16 == 0
+    got = []
+    for path in (0, STREAMING if not streams else CLUSTER if aligned else STREAMING):
+        if parent is None:
+            out = (torch.full((B, 1, call), -9, dtype=torch.int32, device="cuda"), torch.zeros(B, 1, call, device="cuda"))
+            ersd.ersd_race_sample(tgt, seeds, 1.0, out[0], ersd.make_opts(top_c=call, out_key=out[1], kernel_path=path))
+        else:
+            out = (torch.full((B, ersd.ersd_tree_depth(parent) + 1), -9, dtype=torch.int32, device="cuda"),
+                   torch.full((B,), -9, dtype=torch.int32, device="cuda"),
+                   torch.full((B, rows), -9, dtype=torch.int32, device="cuda"))
+            ersd.ersd_verify_tree(tgt, drf, parent, seeds, 1.0, out[0], out[1],
+                                  ersd.make_opts(out_draft_tok=out[2], kernel_path=path))
+        if not got:
+            assert ("ersd_race_kernel" in ersd.ersd_last_launch()) == streams, ersd.ersd_last_launch()
+        got.append(out)
+    torch.cuda.synchronize()
+    assert all((a == b).all() for a, b in zip(*got))
