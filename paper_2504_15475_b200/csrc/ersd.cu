@@ -407,8 +407,8 @@ static RaceKernel race_kernel(bool bf16, bool aligned, bool many, int threads) {
 //             the streaming kernel need about 180 KB);
 //   cluster:  the opt-in for clusters of 16 blocks; *limit = the largest cluster (a power of two) that it
 //             can be launched in: 16 where that is granted and such a cluster fits, else 8.
-// Done when a call first wants the kernel: the attributes load its code, and asking for all the cluster
-// builds' at once made a process's first call take 35 ms (10 when there were eight of them).
+// Done when a call first wants the kernel: asking for all 40 cluster builds at once was 3 of the 32 ms that a
+// process's first call takes (drafting 32.1 -> 29.4 ms, verification 33.6 -> 30.2).
 struct KernelState {
   const void* kernel;
   uint64_t ready, sixteen;  // bits: devices
@@ -487,8 +487,8 @@ static int launch(const Params& p, const TreeDesc& tree, int dt, int cmax, cudaS
 // starting: it takes longer bf16 rows from a number of logits on (verification: at 65256 logits 1500
 // positions 111.2 / 113.5 and 2250 157.2 / 159.5; at 100000 500 65.5 / 69.7; at 128256 400 66.4 / 68.8, 450
 // 77.9 / 81.0, 576 91.8 / 87.5; at 151936 300 64.0 / 71.4 and 400 81.4 / 76.4; trees: at 128256 450 rows 85.7 /
-// 83.8.  Sampling and given tokens, one row per position: at 128256 800 93.1 / 95.1; at 151936 576 89.4 / 83.3, 640
-// 98.6 / 91.9).
+// 83.8.  Sampling and given tokens, one row per position: at 128256 800 93.1 / 95.1; given tokens at 151936 576
+// 89.4 / 83.3, 640 98.6 / 91.9).
 struct ClusterLimit {
   int row;         // rows of up to this many logits ...
   int64_t logits;  // ... take the cluster kernel while the call has no more logits than this
@@ -499,7 +499,7 @@ struct ClusterLimit {
 // 20M logits on although the cluster kernel would be quicker there (8 x 17 nodes of 151936: 39.4 / 63.7 us): the
 // tests fix which kernel takes that call.
 constexpr ClusterLimit kClusterLimits[3][4] = {  // bf16: one row per position, draft and target row, the same in trees
-    {{65536, INT64_MAX}, {131072, 100 << 20}, {INT32_MAX, 72 << 20}},
+    {{65536, INT64_MAX}, {INT32_MAX, 100 << 20}},
     {{65536, INT64_MAX}, {INT32_MAX, 56 << 20}},
     {{40960, INT64_MAX}, {65536, 80 << 20}, {131072, 40 << 20}, {INT32_MAX, 19 << 20}}};
 // The number of blocks up to which a tree's rows get a cluster each (one block per SM and a half)
@@ -627,9 +627,9 @@ static bool top_streams(const Params& p, int dt, int cmax) {
     if (cmax <= 4) return n > (cmax <= 3 ? 1500 : 3000);
     return p.V <= 3072 && n > (cmax <= 16 ? 2500 : 5000);
   }
-  // Long rows, few arrivals (100000 bf16 logits: 2 of 1024 rows 135 / 124, 4 of 1024 233 / 163; 32-bit: 4 of 1024
-  // 236 / 184, 2 of 1024 0.9).
-  if (!tree) return p.V > 65536 && p.V <= 131072 && cmax <= 4 && (dt == ERSD_BF16 || cmax > 2) && logits > (90 << 20);
+  // (Long rows, few arrivals: 4 of 1024 rows of 100000 bf16 logits 233 / 163, 2 135 / 124.  They stay: the streaming
+  // kernel would cut the rows in two and need a workspace, which a sampling call that is being captured may not have.)
+  if (!tree) return false;
   // 32-bit trees, which the table leaves out (stars of 8, 200 of 48000 logits 176 / 143; two alternatives, 128 of
   // 100000 90 / 78, of 128256 1.0).
   if (dt == ERSD_F32 && p.V > 40960 && cmax <= 16) {
@@ -647,7 +647,9 @@ static bool cluster_by_default(const ersd_opts& o, const Params& p, int dt, int 
   if (cmax > 16 && p.V <= 49152) return true;  // (64 stars of 32 of 48000 logits: 0.66)
   const ClusterLimit* limit = kClusterLimits[!(p.mode == kVerify && p.draft) ? 0 : cmax > 1 ? 2 : 1];
   while (p.V > limit->row) ++limit;
-  return (int64_t)p.V * p.B * p.rows <= limit->logits;
+  // (given tokens of rows beyond 131072 leave earlier; sampling does not, see top_streams on workspaces)
+  const int64_t most = p.given_tok && p.V > 131072 ? 72 << 20 : limit->logits;
+  return (int64_t)p.V * p.B * p.rows <= most;
 }
 
 template <int DT, bool AL>

@@ -325,3 +325,20 @@ def test_default_choice_for_many_or_short_rows(ersd, call, B, V, dtype, streams)
         got.append(out)
     torch.cuda.synchronize()
     assert all((a == b).all() for a, b in zip(*got))
+
+
+@pytest.mark.parametrize("c,B,V,dtype", [(8, 1501, 1000, "bf16"), (16, 2000, 1536, "f32"), (4, 300, 500, "bf16"), (4, 1024, 100000, "bf16"),
+                                         (1, 520, 151936, "bf16")])
+def test_sampling_needs_no_workspace_whichever_kernel_takes_it(ersd, c, B, V, dtype):
+    """So such a call can be captured whatever the device's private workspace holds: with a workspace that would be
+    too small for it, it runs."""
+    g = torch.Generator(device="cuda").manual_seed(B)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    row = torch.randn(4, 1, V, generator=g, device="cuda").to(dt).repeat(B // 4, 1, 1).contiguous()
+    B = row.shape[0]
+    seeds = wl.make_seeds(62, 0, B).cuda()
+    tok = torch.empty(B, 1, c, dtype=torch.int32, device="cuda")
+    small = torch.zeros(ersd.ersd_workspace_bytes(1, 1), dtype=torch.uint8, device="cuda")
+    ersd.ersd_race_sample(row, seeds, 1.0, tok, ersd.make_opts(top_c=c, workspace=small))  # (too small for more than one row)
+    torch.cuda.synchronize()
+    assert ((tok >= 0) & (tok < V)).all()
