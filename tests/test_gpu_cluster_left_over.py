@@ -1,0 +1,46 @@
+"""Cluster kernel on staged rows: every warp screens a few of its groups of eight indices, and a row whose
+contenders all belong to one warp, or to one thread, leaves some of them over; those rows are decided by every
+block with the exact key.  Against the CPU oracle."""
+import pytest
+import torch
+
+from paper_2504_15475_b200 import workloads as wl
+
+from parity_util import check_sample, check_verify
+from test_gpu_unaligned_rows import ersd, guarded, inputs  # noqa: F401  (fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+def crowd(z, V):
+    """Rows 0, 4, ..: contenders in the first warp's groups alone; 1, 5, ..: in one thread's groups of all tiles (tiles
+    of 2048 indices that a cluster of 1, 2, 4, 8 or 16 blocks shares out); 2, 6, ..: the row's last group; 3, 7, ..: as drawn."""
+    flat = z.view(-1, V)
+    flat[0::4, :min(V, 256)] += 9.0
+    for i in range(0, V, 2048):
+        flat[1::4, i + 16:i + 24] += 9.0
+    flat[2::4, (V - 1) // 8 * 8:] += 9.0
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("B,V", [(40, 700), (40, 2048), (20, 4100), (10, 16384), (6, 32001), (2, 66000), (1, 131080)])
+def test_contenders_of_one_warp_and_of_one_thread(ersd, B, V, dtype):  # noqa: F811
+    k = 3
+    inp = inputs(B, k, V, "f32")
+    for name in ("target", "draft"):
+        crowd(inp[name], V)
+        inp[name] = wl._storage(inp[name], dtype)
+    on_device = guarded if V % 8 else torch.Tensor.cuda
+    seeds = inp["seeds"].cuda()
+    for T in (0.8, 3.0, 0.0):
+        inp["T"] = T
+        out = ersd.verify(on_device(inp["target"]), on_device(inp["draft"]), seeds, T, want_rows=True)
+        torch.cuda.synchronize()
+        assert "ersd_cluster_kernel" in ersd.ersd_last_launch() and "(unstaged)" not in ersd.ersd_last_launch()
+        check_verify(inp, out)
+        tok = torch.full((B, k + 1, 1), -7, dtype=torch.int32, device="cuda")
+        key = torch.full((B, k + 1, 1), -7.0, dtype=torch.float32, device="cuda")
+        ersd.ersd_race_sample(on_device(inp["target"]), seeds, T, tok, ersd.make_opts(out_key=key))
+        torch.cuda.synchronize()
+        assert "(unstaged)" not in ersd.ersd_last_launch()
+        check_sample(inp["target"], inp["seeds"], T, tok, key)
