@@ -415,7 +415,7 @@ struct KernelState {
 };
 static int prepare_kernel(const void* kernel, size_t smem, bool carveout, bool cluster, int* limit) {
   static std::mutex m;
-  static KernelState known[64];  // (as many as there are builds)
+  static KernelState known[80];  // (no fewer than there are builds)
   static int count;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -426,8 +426,8 @@ static int prepare_kernel(const void* kernel, size_t smem, bool carveout, bool c
   int at = 0;
   while (at < count && known[at].kernel != kernel) ++at;
   KernelState fresh = {kernel, 0, 0};
-  KernelState& k = at < 64 ? known[at] : fresh;
-  if (at == count && at < 64) {
+  KernelState& k = at < 80 ? known[at] : fresh;
+  if (at == count && at < 80) {
     k = fresh;
     ++count;
   }
@@ -515,18 +515,22 @@ static int cluster_max_tiles(int dt, int roles, int cmax, bool aligned) {
 }
 
 // The build of the cluster kernels for rows of type DT, aligned (AL) or not, `roles` of them raced together.
+enum ClusterBuild { kStaged, kUnstaged, kRoomy };
+template <int DT, bool AL, int NR>
+static const void* cluster_kernel(int cmax, ClusterBuild build, bool small) {
+  if (cmax > 1)
+    return build == kStaged ? (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, true> : (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, false>;
+  if (small)
+    return build == kStaged ? (const void*)b128::ersd_cluster_kernel<DT, NR, AL, true, false>
+                            : (const void*)b128::ersd_cluster_kernel<DT, NR, AL, false, false>;
+  if constexpr (DT == ERSD_BF16 && AL && NR == 2)
+    if (build == kRoomy) return (const void*)b256::ersd_cluster_kernel<DT, NR, AL, false, true>;
+  return build == kStaged ? (const void*)b256::ersd_cluster_kernel<DT, NR, AL, true, false>
+                          : (const void*)b256::ersd_cluster_kernel<DT, NR, AL, false, false>;
+}
 template <int DT, bool AL>
-static const void* cluster_kernel(int cmax, int roles, bool staged, bool small) {
-  if (cmax > 1) {
-    if (staged) return roles == 2 ? (const void*)b256::ersd_cluster_top_kernel<DT, 2, AL, true> : (const void*)b256::ersd_cluster_top_kernel<DT, 1, AL, true>;
-    return roles == 2 ? (const void*)b256::ersd_cluster_top_kernel<DT, 2, AL, false> : (const void*)b256::ersd_cluster_top_kernel<DT, 1, AL, false>;
-  }
-  if (small) {
-    if (staged) return roles == 2 ? (const void*)b128::ersd_cluster_kernel<DT, 2, AL, true> : (const void*)b128::ersd_cluster_kernel<DT, 1, AL, true>;
-    return roles == 2 ? (const void*)b128::ersd_cluster_kernel<DT, 2, AL, false> : (const void*)b128::ersd_cluster_kernel<DT, 1, AL, false>;
-  }
-  if (staged) return roles == 2 ? (const void*)b256::ersd_cluster_kernel<DT, 2, AL, true> : (const void*)b256::ersd_cluster_kernel<DT, 1, AL, true>;
-  return roles == 2 ? (const void*)b256::ersd_cluster_kernel<DT, 2, AL, false> : (const void*)b256::ersd_cluster_kernel<DT, 1, AL, false>;
+static const void* cluster_kernel(int cmax, int roles, ClusterBuild build, bool small) {
+  return roles == 2 ? cluster_kernel<DT, AL, 2>(cmax, build, small) : cluster_kernel<DT, AL, 1>(cmax, build, small);
 }
 
 // Whether a call can take a cluster kernel at all; cmax: most arrivals any of its races wants.
@@ -660,7 +664,7 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   int CL = 1;
   const bool staged = cluster_staged(p, DT, roles, cmax);
   int lim = 8;
-  int ls = prepare_kernel(cluster_kernel<DT, AL>(cmax, roles, staged, false), kClusterSmemBytes, false, true, &lim);
+  int ls = prepare_kernel(cluster_kernel<DT, AL>(cmax, roles, staged ? kStaged : kUnstaged, false), kClusterSmemBytes, false, true, &lim);
   if (ls == ERSD_OK) ls = cluster_size(o, p, DT, cmax, staged, lim, &CL);
   if (ls != ERSD_OK) return ls;
   const int ntiles = (p.V + b256::kTile - 1) / b256::kTile;
@@ -679,7 +683,7 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
       split = true;
     }
     if (split) {
-      ls = prepare_kernel(cluster_kernel<DT, AL>(cmax, 1, staged, false), kClusterSmemBytes, false, true, &lim);
+      ls = prepare_kernel(cluster_kernel<DT, AL>(cmax, 1, staged ? kStaged : kUnstaged, false), kClusterSmemBytes, false, true, &lim);
       if (ls != ERSD_OK) return ls;
     }
     if (split && CL <= lim) {
@@ -712,10 +716,13 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   snprintf(g_last_launch, sizeof g_last_launch, "%s<%s, %d row(s) per cluster>: %d clusters of %d x %d threads, %d positions%s",
            cmax > 1 ? "ersd_cluster_top_kernel" : "ersd_cluster_kernel", DT == ERSD_BF16 ? "bf16" : "f32", roles,
            p.B * jobs, CL, threads, p.B * p.rows, staged ? "" : " (unstaged)");
-  const void* kernel = cluster_kernel<DT, AL>(cmax, roles, staged, small);
-  if (small) {  // (the other builds are prepared by now)
-    ls = prepare_kernel(kernel, staged ? kClusterSmemBytes : 0, false, false, nullptr);
+  // Up to three blocks to an SM: the build that asks for three tiles ahead (see cluster_ahead).
+  const bool roomy = DT == ERSD_BF16 && AL && roles == 2 && cmax == 1 && !staged && !small && (int64_t)CL * jobs * p.B <= 3 * sm_count();
+  const void* kernel = cluster_kernel<DT, AL>(cmax, roles, staged ? kStaged : roomy ? kRoomy : kUnstaged, small);
+  if (small || roomy) {  // (the other builds are prepared by now)
+    ls = prepare_kernel(kernel, staged || roomy ? kClusterSmemBytes : 0, false, roomy, &lim);
     if (ls != ERSD_OK) return ls;
+    if (CL > lim) return ERSD_EUNSUPPORTED;
   }
   void* args[] = {&p, const_cast<TreeDesc*>(&tree)};  // (the kernel for one arrival has the first alone)
   const cudaError_t e = cudaLaunchKernelExC(&l.cfg, kernel, args);
