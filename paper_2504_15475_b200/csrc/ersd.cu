@@ -515,22 +515,24 @@ static int cluster_max_tiles(int dt, int roles, int cmax, bool aligned) {
 }
 
 // The build of the cluster kernels for rows of type DT, aligned (AL) or not, `roles` of them raced together.
-enum ClusterBuild { kStaged, kUnstaged, kRoomy };
+// short_way: ersd_cluster_kernel's build that asks for more tiles ahead, ersd_cluster_top_kernel's DIRECT build.
 template <int DT, bool AL, int NR>
-static const void* cluster_kernel(int cmax, ClusterBuild build, bool small) {
-  if (cmax > 1)
-    return build == kStaged ? (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, true> : (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, false>;
+static const void* cluster_kernel(int cmax, bool staged, bool small, bool short_way) {
+  if (cmax > 1) {
+    if constexpr (NR == 1)
+      if (short_way)
+        return staged ? (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, true, true> : (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, false, true>;
+    return staged ? (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, true, false> : (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, false, false>;
+  }
   if (small)
-    return build == kStaged ? (const void*)b128::ersd_cluster_kernel<DT, NR, AL, true, false>
-                            : (const void*)b128::ersd_cluster_kernel<DT, NR, AL, false, false>;
+    return staged ? (const void*)b128::ersd_cluster_kernel<DT, NR, AL, true, false> : (const void*)b128::ersd_cluster_kernel<DT, NR, AL, false, false>;
   if constexpr (DT == ERSD_BF16 && AL && NR == 2)
-    if (build == kRoomy) return (const void*)b256::ersd_cluster_kernel<DT, NR, AL, false, true>;
-  return build == kStaged ? (const void*)b256::ersd_cluster_kernel<DT, NR, AL, true, false>
-                          : (const void*)b256::ersd_cluster_kernel<DT, NR, AL, false, false>;
+    if (short_way) return (const void*)b256::ersd_cluster_kernel<DT, NR, AL, false, true>;
+  return staged ? (const void*)b256::ersd_cluster_kernel<DT, NR, AL, true, false> : (const void*)b256::ersd_cluster_kernel<DT, NR, AL, false, false>;
 }
 template <int DT, bool AL>
-static const void* cluster_kernel(int cmax, int roles, ClusterBuild build, bool small) {
-  return roles == 2 ? cluster_kernel<DT, AL, 2>(cmax, build, small) : cluster_kernel<DT, AL, 1>(cmax, build, small);
+static const void* cluster_kernel(int cmax, int roles, bool staged, bool small, bool short_way) {
+  return roles == 2 ? cluster_kernel<DT, AL, 2>(cmax, staged, small, short_way) : cluster_kernel<DT, AL, 1>(cmax, staged, small, short_way);
 }
 
 // Whether a call can take a cluster kernel at all; cmax: most arrivals any of its races wants.
@@ -664,7 +666,7 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   int CL = 1;
   const bool staged = cluster_staged(p, DT, roles, cmax);
   int lim = 8;
-  int ls = prepare_kernel(cluster_kernel<DT, AL>(cmax, roles, staged ? kStaged : kUnstaged, false), kClusterSmemBytes, false, true, &lim);
+  int ls = prepare_kernel(cluster_kernel<DT, AL>(cmax, roles, staged, false, false), kClusterSmemBytes, false, true, &lim);
   if (ls == ERSD_OK) ls = cluster_size(o, p, DT, cmax, staged, lim, &CL);
   if (ls != ERSD_OK) return ls;
   const int ntiles = (p.V + b256::kTile - 1) / b256::kTile;
@@ -683,7 +685,7 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
       split = true;
     }
     if (split) {
-      ls = prepare_kernel(cluster_kernel<DT, AL>(cmax, 1, staged ? kStaged : kUnstaged, false), kClusterSmemBytes, false, true, &lim);
+      ls = prepare_kernel(cluster_kernel<DT, AL>(cmax, 1, staged, false, false), kClusterSmemBytes, false, true, &lim);
       if (ls != ERSD_OK) return ls;
     }
     if (split && CL <= lim) {
@@ -716,13 +718,20 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   snprintf(g_last_launch, sizeof g_last_launch, "%s<%s, %d row(s) per cluster>: %d clusters of %d x %d threads, %d positions%s",
            cmax > 1 ? "ersd_cluster_top_kernel" : "ersd_cluster_kernel", DT == ERSD_BF16 ? "bf16" : "f32", roles,
            p.B * jobs, CL, threads, p.B * p.rows, staged ? "" : " (unstaged)");
-  // Up to three blocks to an SM: the build that asks for three tiles ahead (see cluster_ahead).
-  const bool roomy = DT == ERSD_BF16 && AL && roles == 2 && cmax == 1 && !staged && !small && (int64_t)CL * jobs * p.B <= 3 * sm_count();
-  const void* kernel = cluster_kernel<DT, AL>(cmax, roles, staged ? kStaged : roomy ? kRoomy : kUnstaged, small);
-  if (small || roomy) {  // (the other builds are prepared by now)
-    ls = prepare_kernel(kernel, staged || roomy ? kClusterSmemBytes : 0, false, roomy, &lim);
+  // Builds for some calls (where the device does not take them in clusters of this size: the general one).  Pairs of
+  // rows in up to three blocks to an SM: see cluster_ahead.  Several arrivals, with ten warps of the cluster to an
+  // arrival: see DIRECT.
+  bool short_way = cmax == 1 ? DT == ERSD_BF16 && AL && roles == 2 && !staged && !small && (int64_t)CL * jobs * p.B <= 3 * sm_count()
+                             : roles == 1 && CL * b256::kWarps >= 10 * cmax;
+  if (short_way) {
+    ls = prepare_kernel(cluster_kernel<DT, AL>(cmax, roles, staged, small, true), kClusterSmemBytes, false, true, &lim);
     if (ls != ERSD_OK) return ls;
-    if (CL > lim) return ERSD_EUNSUPPORTED;
+    short_way = CL <= lim;
+  }
+  const void* kernel = cluster_kernel<DT, AL>(cmax, roles, staged, small, short_way);
+  if (small) {  // (the other builds are prepared by now)
+    ls = prepare_kernel(kernel, staged ? kClusterSmemBytes : 0, false, false, nullptr);
+    if (ls != ERSD_OK) return ls;
   }
   void* args[] = {&p, const_cast<TreeDesc*>(&tree)};  // (the kernel for one arrival has the first alone)
   const cudaError_t e = cudaLaunchKernelExC(&l.cfg, kernel, args);

@@ -44,3 +44,45 @@ def test_contenders_of_one_warp_and_of_one_thread(ersd, B, V, dtype):  # noqa: F
         torch.cuda.synchronize()
         assert "(unstaged)" not in ersd.ersd_last_launch()
         check_sample(inp["target"], inp["seeds"], T, tok, key)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("B,V,c", [(4, 131072, 2), (2, 100001, 4), (1, 131080, 8), (4, 128256, 12), (1, 40961, 5), (40, 70001, 4),
+                                   (30, 128256, 3)])
+def test_several_arrivals_of_one_warp_and_of_one_thread(ersd, B, V, c, dtype):  # noqa: F811
+    """Staged and not; rows of ties, rows with fewer tokens than arrivals, infinities, and rows as drawn."""
+    inp = inputs(2 * B, 0, V, "f32")
+    z = inp["target"]
+    crowd(z, V)
+    flat = z.view(-1, V)
+    if B > 1:
+        flat[B] = 0.5                        # under T = 0 a tie of the whole row
+        flat[B + 1, 3:] = float("-inf")      # three tokens
+    if B > 3:
+        flat[B + 2, V - 1] = float("inf")
+        flat[B + 3] = (flat[B + 3] * 2).round() / 2
+    z = wl._storage(z, dtype)
+    on_device = guarded if V % 8 else torch.Tensor.cuda
+    for T in (0.8, 2.5, 0.0):
+        tok = torch.full((2 * B, 1, c), -7, dtype=torch.int32, device="cuda")
+        key = torch.full((2 * B, 1, c), -7.0, dtype=torch.float32, device="cuda")
+        ersd.ersd_race_sample(on_device(z), inp["seeds"].cuda(), T, tok, ersd.make_opts(top_c=c, out_key=key))
+        torch.cuda.synchronize()
+        assert "ersd_cluster_top_kernel" in ersd.ersd_last_launch()
+        check_sample(z, inp["seeds"], T, tok, key, c=c)
+
+
+@pytest.mark.parametrize("name", ["specinfer", "4x4"])
+def test_trees_whose_rows_have_a_cluster_each(ersd, name):  # noqa: F811
+    parent = {"specinfer": wl.TREE_SPECINFER, "4x4": wl.TREE_4x4}[name]
+    for V, T in ((128256, 0.8), (70001, 3.0), (40000, 0.0)):
+        inp = inputs(1, len(parent) - 1, V, "f32", parent=parent)
+        inp["T"] = T
+        for n in ("target", "draft"):
+            crowd(inp[n], V)
+            inp[n] = wl._storage(inp[n], "bf16")
+        on_device = guarded if V % 8 else torch.Tensor.cuda
+        out = ersd.verify(on_device(inp["target"]), on_device(inp["draft"]), inp["seeds"].cuda(), T, want_rows=True, parent=list(parent))
+        torch.cuda.synchronize()
+        assert "ersd_cluster_top_kernel" in ersd.ersd_last_launch()
+        check_verify(inp, out)
