@@ -415,7 +415,7 @@ struct KernelState {
 };
 static int prepare_kernel(const void* kernel, size_t smem, bool carveout, bool cluster, int* limit) {
   static std::mutex m;
-  static KernelState known[80];  // (no fewer than there are builds)
+  static KernelState known[96];  // (no fewer than there are builds)
   static int count;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -426,8 +426,8 @@ static int prepare_kernel(const void* kernel, size_t smem, bool carveout, bool c
   int at = 0;
   while (at < count && known[at].kernel != kernel) ++at;
   KernelState fresh = {kernel, 0, 0};
-  KernelState& k = at < 80 ? known[at] : fresh;
-  if (at == count && at < 80) {
+  KernelState& k = at < 96 ? known[at] : fresh;
+  if (at == count && at < 96) {
     k = fresh;
     ++count;
   }
@@ -515,7 +515,7 @@ static int cluster_max_tiles(int dt, int roles, int cmax, bool aligned) {
 }
 
 // The build of the cluster kernels for rows of type DT, aligned (AL) or not, `roles` of them raced together.
-// short_way: ersd_cluster_kernel's build that asks for more tiles ahead, ersd_cluster_top_kernel's DIRECT build.
+// short_way: the FAST builds of ersd_cluster_kernel, the DIRECT builds of ersd_cluster_top_kernel.
 template <int DT, bool AL, int NR>
 static const void* cluster_kernel(int cmax, bool staged, bool small, bool short_way) {
   if (cmax > 1) {
@@ -526,9 +526,11 @@ static const void* cluster_kernel(int cmax, bool staged, bool small, bool short_
   }
   if (small)
     return staged ? (const void*)b128::ersd_cluster_kernel<DT, NR, AL, true, false> : (const void*)b128::ersd_cluster_kernel<DT, NR, AL, false, false>;
+  if (staged)
+    return short_way ? (const void*)b256::ersd_cluster_kernel<DT, NR, AL, true, true> : (const void*)b256::ersd_cluster_kernel<DT, NR, AL, true, false>;
   if constexpr (DT == ERSD_BF16 && AL && NR == 2)
     if (short_way) return (const void*)b256::ersd_cluster_kernel<DT, NR, AL, false, true>;
-  return staged ? (const void*)b256::ersd_cluster_kernel<DT, NR, AL, true, false> : (const void*)b256::ersd_cluster_kernel<DT, NR, AL, false, false>;
+  return (const void*)b256::ersd_cluster_kernel<DT, NR, AL, false, false>;
 }
 template <int DT, bool AL>
 static const void* cluster_kernel(int cmax, int roles, bool staged, bool small, bool short_way) {
@@ -718,11 +720,12 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   snprintf(g_last_launch, sizeof g_last_launch, "%s<%s, %d row(s) per cluster>: %d clusters of %d x %d threads, %d positions%s",
            cmax > 1 ? "ersd_cluster_top_kernel" : "ersd_cluster_kernel", DT == ERSD_BF16 ? "bf16" : "f32", roles,
            p.B * jobs, CL, threads, p.B * p.rows, staged ? "" : " (unstaged)");
-  // Builds for some calls (where the device does not take them in clusters of this size: the general one).  Pairs of
-  // rows in up to three blocks to an SM: see cluster_ahead.  Several arrivals, with ten warps of the cluster to an
-  // arrival: see DIRECT.
-  bool short_way = cmax == 1 ? DT == ERSD_BF16 && AL && roles == 2 && !staged && !small && (int64_t)CL * jobs * p.B <= 3 * sm_count()
-                             : roles == 1 && CL * b256::kWarps >= 10 * cmax;
+  // Builds for some calls (where the device does not take them in clusters of this size: the general one).  Staged rows
+  // in clusters of at least four blocks: the short way of ersd_cluster_kernel.  Unstaged pairs of rows in up to three
+  // blocks to an SM: see cluster_ahead.  Several arrivals, with ten warps of the cluster to an arrival: see DIRECT.
+  bool short_way = cmax > 1 ? roles == 1 && CL * b256::kWarps >= 10 * cmax
+                   : staged ? CL >= 4
+                            : DT == ERSD_BF16 && AL && roles == 2 && !small && (int64_t)CL * jobs * p.B <= 3 * sm_count();
   if (short_way) {
     ls = prepare_kernel(cluster_kernel<DT, AL>(cmax, roles, staged, small, true), kClusterSmemBytes, false, true, &lim);
     if (ls != ERSD_OK) return ls;
