@@ -5,10 +5,9 @@
 // shared-memory ring filled by cp.async; per group of eight vocabulary indices
 // a thread draws the Philox words and compares one cheap lower bound of the
 // eight race keys with the block's running threshold.  The few groups that
-// survive are screened index by index in single precision; the survivors of
-// that are noted and decided in double precision at the chunk's end (races of
-// several arrivals in calls of few rows: at once, in per-warp sorted lists).
-// Results are merged per block, exchanged through a small workspace, and the
+// survive are screened index by index in single precision and the survivors of
+// that are decided in double precision and kept in per-warp sorted lists.
+// Lists are merged per block, exchanged through a small workspace, and the
 // last block of a sequence turns the winners into the accepted prefix
 // (sequence scan or tree walk) in the same launch.
 #include <cuda_runtime.h>

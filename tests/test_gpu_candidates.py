@@ -1,13 +1,12 @@
-"""Streaming kernel, races of up to 32 arrivals: what a warp notes until its chunk ends has limited room, and rows
-on which screening cannot tell the indices apart (equal logits under T = 0, logits so large that single
-precision cannot tell their keys apart) overflow it.  Against the CPU oracle."""
+"""Streaming kernel in calls of many rows, on rows on which screening cannot tell the indices apart: equal logits under
+T = 0, logits so large that single precision cannot tell their keys apart.  Against the CPU oracle."""
 import pytest
 import torch
 
 from paper_2504_15475_b200 import workloads as wl
 
-from parity_util import check_sample
-from test_gpu_unaligned_rows import ersd  # noqa: F401  (fixture)
+from parity_util import check_sample, check_verify
+from test_gpu_unaligned_rows import ersd, inputs  # noqa: F401  (fixture)
 
 pytestmark = pytest.mark.gpu
 
@@ -37,3 +36,26 @@ def test_more_ties_than_a_warp_has_room_for(ersd, c, threads, split):  # noqa: F
     torch.cuda.synchronize()
     assert "ersd_race_kernel" in ersd.ersd_last_launch() and "pooled" not in ersd.ersd_last_launch()
     check_sample(z, seeds, 1.0, tok, None, c=c, temps=temps.numpy())
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("threads", [128, 256])
+def test_ties_in_both_rows_of_a_node(ersd, threads, dtype):  # noqa: F811
+    """Trees of more than two rows per SM, aligned rows: ties in a node's target row, in its draft row, and in both."""
+    parent, B, V = [-1, 0, 0, 0, 1, 1], 80, 5000
+    inp = inputs(B, len(parent) - 1, V, "f32", parent=parent)
+    inp["T"] = 0.0
+    for b in range(0, B, 8):
+        for name in ("target", "draft"):
+            inp[name][b] = 0.25                                               # both rows of every node
+            inp[name][b + 1, :, 3000:] = 9.0
+            inp[name][b + 2, :, ::7] = float("inf")
+        inp["target"][b + 3] = inp["draft"][b + 4] = -1.5                     # one of them
+        inp["draft"][b + 5, :, 2:] = float("-inf")                            # fewer tokens than children
+    for name in ("target", "draft"):
+        inp[name] = wl._storage(inp[name], dtype)
+    out = ersd.verify(inp["target"].cuda(), inp["draft"].cuda(), inp["seeds"].cuda(), 0.0, want_rows=True, parent=parent,
+                      kernel_path=1, block_threads=threads)
+    torch.cuda.synchronize()
+    assert "ersd_race_kernel" in ersd.ersd_last_launch() and "pooled" not in ersd.ersd_last_launch()
+    assert check_verify(inp, out) == 0  # (greedy keys are exact: ties go to the lowest id)
