@@ -180,7 +180,7 @@ __global__ void ersd_row_keys_kernel(const void* row, int V, float T, uint64_t s
 // host side
 // ---------------------------------------------------------------------------------------------
 static thread_local int g_last_cuda_error = 0;
-static thread_local char g_last_launch[160] = "";  // ersd_last_launch(): what this thread's last call launched
+static thread_local char g_last_launch[192] = "";  // ersd_last_launch(): what this thread's last call launched
 
 // The error stays with the library: the runtime keeps it per thread too, where the next check of some
 // other launch on this thread would find it.
@@ -717,9 +717,6 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   // blocks, 9.1 and 8.1, 300 positions of 8192 logits 12.9 and 11.0, and the streaming kernel, two
   // blocks to an SM, 47.5 and 38.9.)
   p.early = (int64_t)CL * jobs * p.B <= (cmax > 1 ? 2 : 1) * sm_count();
-  snprintf(g_last_launch, sizeof g_last_launch, "%s<%s, %d row(s) per cluster>: %d clusters of %d x %d threads, %d positions%s",
-           cmax > 1 ? "ersd_cluster_top_kernel" : "ersd_cluster_kernel", DT == ERSD_BF16 ? "bf16" : "f32", roles,
-           p.B * jobs, CL, threads, p.B * p.rows, staged ? "" : " (unstaged)");
   // Builds for some calls (where the device does not take them in clusters of this size: the general one).  Staged rows
   // in clusters of at least four blocks: the short way of ersd_cluster_kernel.  Unstaged pairs of rows in up to three
   // blocks to an SM: see cluster_ahead.  Several arrivals, with ten warps of the cluster to an arrival: see DIRECT.
@@ -731,6 +728,10 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
     if (ls != ERSD_OK) return ls;
     short_way = CL <= lim;
   }
+  snprintf(g_last_launch, sizeof g_last_launch, "%s<%s, %d row(s) per cluster>: %d clusters of %d x %d threads, %d positions%s%s",
+           cmax > 1 ? "ersd_cluster_top_kernel" : "ersd_cluster_kernel", DT == ERSD_BF16 ? "bf16" : "f32", roles,
+           p.B * jobs, CL, threads, p.B * p.rows, staged ? "" : " (unstaged)",
+           !short_way ? "" : cmax == 1 && !staged ? ", more tiles ahead" : ", short way");
   const void* kernel = cluster_kernel<DT, AL>(cmax, roles, staged, small, short_way);
   if (small) {  // (the other builds are prepared by now)
     ls = prepare_kernel(kernel, staged ? kClusterSmemBytes : 0, false, false, nullptr);

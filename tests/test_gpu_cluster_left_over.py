@@ -1,6 +1,7 @@
-"""Cluster kernel on staged rows: every warp screens a few of its groups of eight indices, and a row whose
-contenders all belong to one warp, or to one thread, leaves some of them over; those rows are decided by every
-block with the exact key.  Against the CPU oracle."""
+"""Cluster kernels' short ways: every warp screens a few of its groups of eight indices, and a row whose
+contenders all belong to one warp, or to one thread, leaves some of them over; those rows are decided the long
+way (one arrival: by every block, with the exact key).  Calls that do not take the short way race the same
+rows.  Against the CPU oracle."""
 import pytest
 import torch
 
@@ -23,9 +24,11 @@ def crowd(z, V):
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
-@pytest.mark.parametrize("B,V", [(40, 700), (40, 2048), (20, 4100), (10, 16384), (6, 32001), (2, 66000), (1, 131080)])
+@pytest.mark.parametrize("B,V", [(40, 700), (40, 2048), (20, 4100), (10, 16384), (6, 32001), (2, 66000), (1, 131080),
+                                 (2, 66001), (6, 33001), (4, 50001)])
 def test_contenders_of_one_warp_and_of_one_thread(ersd, B, V, dtype):  # noqa: F811
-    k = 3
+    """Clusters of one or two blocks (the long way), of four, eight and sixteen."""
+    k, short = 3, V > 16384
     inp = inputs(B, k, V, "f32")
     for name in ("target", "draft"):
         crowd(inp[name], V)
@@ -37,18 +40,19 @@ def test_contenders_of_one_warp_and_of_one_thread(ersd, B, V, dtype):  # noqa: F
         out = ersd.verify(on_device(inp["target"]), on_device(inp["draft"]), seeds, T, want_rows=True)
         torch.cuda.synchronize()
         assert "ersd_cluster_kernel" in ersd.ersd_last_launch() and "(unstaged)" not in ersd.ersd_last_launch()
+        assert ("short way" in ersd.ersd_last_launch()) == short
         check_verify(inp, out)
         tok = torch.full((B, k + 1, 1), -7, dtype=torch.int32, device="cuda")
         key = torch.full((B, k + 1, 1), -7.0, dtype=torch.float32, device="cuda")
         ersd.ersd_race_sample(on_device(inp["target"]), seeds, T, tok, ersd.make_opts(out_key=key))
         torch.cuda.synchronize()
-        assert "(unstaged)" not in ersd.ersd_last_launch()
+        assert "(unstaged)" not in ersd.ersd_last_launch() and ("short way" in ersd.ersd_last_launch()) == short
         check_sample(inp["target"], inp["seeds"], T, tok, key)
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("B,V,c", [(4, 131072, 2), (2, 100001, 4), (1, 131080, 8), (4, 128256, 12), (1, 40961, 5), (40, 70001, 4),
-                                   (30, 128256, 3)])
+                                   (30, 128256, 3), (30, 100001, 2)])
 def test_several_arrivals_of_one_warp_and_of_one_thread(ersd, B, V, c, dtype):  # noqa: F811
     """Staged and not; rows of ties, rows with fewer tokens than arrivals, infinities, and rows as drawn."""
     inp = inputs(2 * B, 0, V, "f32")
@@ -69,6 +73,7 @@ def test_several_arrivals_of_one_warp_and_of_one_thread(ersd, B, V, c, dtype):  
         ersd.ersd_race_sample(on_device(z), inp["seeds"].cuda(), T, tok, ersd.make_opts(top_c=c, out_key=key))
         torch.cuda.synchronize()
         assert "ersd_cluster_top_kernel" in ersd.ersd_last_launch()
+        assert ("short way" in ersd.ersd_last_launch()) == (B < 40)  # (80 rows get clusters of 32 warps: too few for 4 arrivals)
         check_sample(z, inp["seeds"], T, tok, key, c=c)
 
 
@@ -85,4 +90,5 @@ def test_trees_whose_rows_have_a_cluster_each(ersd, name):  # noqa: F811
         out = ersd.verify(on_device(inp["target"]), on_device(inp["draft"]), inp["seeds"].cuda(), T, want_rows=True, parent=list(parent))
         torch.cuda.synchronize()
         assert "ersd_cluster_top_kernel" in ersd.ersd_last_launch()
+        assert ("1 row(s) per cluster" in ersd.ersd_last_launch()) == ("short way" in ersd.ersd_last_launch()), ersd.ersd_last_launch()
         check_verify(inp, out)

@@ -42,6 +42,17 @@ def test_against_the_oracle(ersd, positions, V, dtype):  # noqa: F811
         check_sample(logits, seeds, 0.8, tok, key)
 
 
+@pytest.mark.parametrize("positions,V", [(20, 128256), (100, 128256), (96, 40960), (48, 65544), (112, 24584)])
+def test_three_tiles_ahead(ersd, positions, V):  # noqa: F811
+    """Aligned pairs of bf16 rows, up to three blocks to an SM: 5 to 16 tiles to a block, whole and ragged."""
+    inp = inputs(positions // 2, 1, V, "bf16")
+    out = ersd.verify(inp["target"].cuda(), inp["draft"].cuda(), inp["seeds"].cuda(), inp["T"], want_rows=True)
+    torch.cuda.synchronize()
+    unstaged(ersd)
+    assert "more tiles ahead" in ersd.ersd_last_launch(), ersd.ersd_last_launch()
+    check_verify(inp, out)
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 def test_special_values_as_in_the_streaming_kernel(ersd, dtype):  # noqa: F811
     V, B = 5000, 160
