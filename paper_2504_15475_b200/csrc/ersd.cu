@@ -528,7 +528,7 @@ static const void* cluster_kernel(int cmax, bool staged, bool small, bool short_
     return staged ? (const void*)b128::ersd_cluster_kernel<DT, NR, AL, true, false> : (const void*)b128::ersd_cluster_kernel<DT, NR, AL, false, false>;
   if (staged)
     return short_way ? (const void*)b256::ersd_cluster_kernel<DT, NR, AL, true, true> : (const void*)b256::ersd_cluster_kernel<DT, NR, AL, true, false>;
-  if constexpr (DT == ERSD_BF16 && AL && NR == 2)
+  if constexpr (NR == 2 ? DT == ERSD_BF16 && AL : DT == ERSD_F32)
     if (short_way) return (const void*)b256::ersd_cluster_kernel<DT, NR, AL, false, true>;
   return (const void*)b256::ersd_cluster_kernel<DT, NR, AL, false, false>;
 }
@@ -711,18 +711,21 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   const size_t smem = (small ? b128::cluster_role_bytes<DT>(G, AL, staged) : b256::cluster_role_bytes<DT>(G, AL, staged)) * (size_t)roles +
                       (cmax > 1 ? b256::top_list_bytes(cmax, CL) : 0);
   Launch l(dim3((unsigned)CL, (unsigned)jobs, (unsigned)p.B), (unsigned)threads, smem, st, (unsigned)CL);
+  const int64_t blocks = (int64_t)CL * jobs * p.B;
   // The next kernel's blocks go where this one's leave room: if this one has a block on every SM they
   // are spread unevenly when they start early.  (One row of 128256 logits 4.8 us with it and 5.0
   // without, 4 x 8 alternatives 10.7 and 11.6, a tree of 240 blocks 21.1 and 22.1; but 16 rows, 256
   // blocks, 9.1 and 8.1, 300 positions of 8192 logits 12.9 and 11.0, and the streaming kernel, two
   // blocks to an SM, 47.5 and 38.9.)
-  p.early = (int64_t)CL * jobs * p.B <= (cmax > 1 ? 2 : 1) * sm_count();
+  p.early = blocks <= (cmax > 1 ? 2 : 1) * sm_count();
   // Builds for some calls (where the device does not take them in clusters of this size: the general one).  Staged rows
-  // in clusters of at least four blocks: the short way of ersd_cluster_kernel.  Unstaged pairs of rows in up to three
-  // blocks to an SM: see cluster_ahead.  Several arrivals, with ten warps of the cluster to an arrival: see DIRECT.
-  bool short_way = cmax > 1 ? roles == 1 && CL * b256::kWarps >= 10 * cmax
-                   : staged ? CL >= 4
-                            : DT == ERSD_BF16 && AL && roles == 2 && !small && (int64_t)CL * jobs * p.B <= 3 * sm_count();
+  // in clusters of at least four blocks: the short way of ersd_cluster_kernel.  Unstaged rows, by blocks to an SM: see
+  // cluster_ahead.  Several arrivals, with ten warps of the cluster to an arrival: see DIRECT.
+  bool short_way = cmax > 1     ? roles == 1 && CL * b256::kWarps >= 10 * cmax
+                   : staged     ? CL >= 4
+                   : small      ? false
+                   : roles == 2 ? DT == ERSD_BF16 && AL && blocks <= 3 * sm_count()
+                                : DT == ERSD_F32 && blocks > 3 * sm_count() && G > 16;
   if (short_way) {
     ls = prepare_kernel(cluster_kernel<DT, AL>(cmax, roles, staged, small, true), kClusterSmemBytes, false, true, &lim);
     if (ls != ERSD_OK) return ls;

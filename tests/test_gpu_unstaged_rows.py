@@ -53,6 +53,22 @@ def test_three_tiles_ahead(ersd, positions, V):  # noqa: F811
     check_verify(inp, out)
 
 
+@pytest.mark.parametrize("rows,V,more", [(100, 32000, False), (450, 34816, True), (450, 34817, True), (450, 32768, False), (300, 38912, False),
+                                         (150, 151936, True), (230, 69640, True)])
+def test_32_bit_rows_two_tiles_ahead(ersd, rows, V, more):  # noqa: F811
+    """One row per position: 17 tiles to a block and more, in more than three blocks to an SM."""
+    logits = inputs(rows, 0, V, "f32")["target"]
+    seeds = wl.make_seeds(7, V, rows)
+    tok = torch.full((rows, 1, 1), -7, dtype=torch.int32, device="cuda")
+    key = torch.full((rows, 1, 1), -7.0, dtype=torch.float32, device="cuda")
+    on_device = guarded if V % 8 else torch.Tensor.cuda
+    ersd.ersd_race_sample(on_device(logits), seeds.cuda(), 0.8, tok, ersd.make_opts(out_key=key))
+    torch.cuda.synchronize()
+    unstaged(ersd)
+    assert ("more tiles ahead" in ersd.ersd_last_launch()) == more, ersd.ersd_last_launch()
+    check_sample(logits, seeds, 0.8, tok, key)
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 def test_special_values_as_in_the_streaming_kernel(ersd, dtype):  # noqa: F811
     V, B = 5000, 160
