@@ -720,8 +720,8 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   p.early = blocks <= (cmax > 1 ? 2 : 1) * sm_count();
   // Builds for some calls (where the device does not take them in clusters of this size: the general one).  Staged rows
   // in clusters of at least four blocks: the short way of ersd_cluster_kernel.  Unstaged rows, by blocks to an SM: see
-  // cluster_ahead.  Several arrivals, with ten warps of the cluster to an arrival: see DIRECT.
-  bool short_way = cmax > 1     ? roles == 1 && CL * b256::kWarps >= 10 * cmax
+  // cluster_ahead.  Several arrivals, with ten warps of the cluster to an arrival, unless all rows are greedy: see DIRECT.
+  bool short_way = cmax > 1     ? roles == 1 && CL * b256::kWarps >= 10 * cmax && (p.temps || p.T != 0.0f)
                    : staged     ? CL >= 4
                    : small      ? false
                    : roles == 2 ? DT == ERSD_BF16 && AL && blocks <= 3 * sm_count()

@@ -73,8 +73,26 @@ def test_several_arrivals_of_one_warp_and_of_one_thread(ersd, B, V, c, dtype):  
         ersd.ersd_race_sample(on_device(z), inp["seeds"].cuda(), T, tok, ersd.make_opts(top_c=c, out_key=key))
         torch.cuda.synchronize()
         assert "ersd_cluster_top_kernel" in ersd.ersd_last_launch()
-        assert ("short way" in ersd.ersd_last_launch()) == (B < 40)  # (80 rows get clusters of 32 warps: too few for 4 arrivals)
+        # (80 rows get clusters of 32 warps: too few for four arrivals; greedy calls go the long way)
+        assert ("short way" in ersd.ersd_last_launch()) == (B < 40 and T > 0)
         check_sample(z, inp["seeds"], T, tok, key, c=c)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_greedy_rows_among_others(ersd, dtype):  # noqa: F811
+    """A call whose rows have temperatures of their own takes the short way's build, in which greedy rows go the long way."""
+    B, V, c = 12, 100008, 4
+    z = inputs(B, 0, V, "f32")["target"]
+    crowd(z, V)
+    z[8:] = (z[8:] * 2).round() / 2
+    temps = torch.tensor([0.8, 0.0]).repeat(B // 2).view(B, 1).contiguous()
+    z, seeds = wl._storage(z, dtype), wl.make_seeds(31, c, B)
+    tok = torch.full((B, 1, c), -7, dtype=torch.int32, device="cuda")
+    key = torch.full((B, 1, c), -7.0, dtype=torch.float32, device="cuda")
+    ersd.ersd_race_sample(z.cuda(), seeds.cuda(), 1.0, tok, ersd.make_opts(top_c=c, out_key=key, temps=temps.cuda(), temp_strides=(1, 1)))
+    torch.cuda.synchronize()
+    assert "ersd_cluster_top_kernel" in ersd.ersd_last_launch() and "short way" in ersd.ersd_last_launch()
+    check_sample(z, seeds, 1.0, tok, key, c=c, temps=temps.numpy())
 
 
 @pytest.mark.parametrize("name", ["specinfer", "4x4"])
@@ -90,5 +108,5 @@ def test_trees_whose_rows_have_a_cluster_each(ersd, name):  # noqa: F811
         out = ersd.verify(on_device(inp["target"]), on_device(inp["draft"]), inp["seeds"].cuda(), T, want_rows=True, parent=list(parent))
         torch.cuda.synchronize()
         assert "ersd_cluster_top_kernel" in ersd.ersd_last_launch()
-        assert ("1 row(s) per cluster" in ersd.ersd_last_launch()) == ("short way" in ersd.ersd_last_launch()), ersd.ersd_last_launch()
+        assert "1 row(s) per cluster" in ersd.ersd_last_launch() and ("short way" in ersd.ersd_last_launch()) == (T > 0)
         check_verify(inp, out)
