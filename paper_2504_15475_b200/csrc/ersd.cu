@@ -517,12 +517,14 @@ static int cluster_max_tiles(int dt, int roles, int cmax, bool aligned) {
 // The build of the cluster kernels for rows of type DT, aligned (AL) or not, `roles` of them raced together.
 // short_way: the FAST builds of ersd_cluster_kernel, the DIRECT builds of ersd_cluster_top_kernel.
 template <int DT, bool AL, int NR>
-static const void* cluster_kernel(int cmax, bool staged, bool small, bool short_way) {
+static const void* cluster_kernel(bool verify, int cmax, bool staged, bool small, bool short_way) {
   if (cmax > 1) {
-    if constexpr (NR == 1)
+    if constexpr (NR == 1) {
       if (short_way)
-        return staged ? (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, true, true> : (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, false, true>;
-    return staged ? (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, true, false> : (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, false, false>;
+        return staged ? (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, true, true, true> : (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, false, true, true>;
+      if (!staged && !verify) return (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, false, false, false>;
+    }
+    return staged ? (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, true, false, true> : (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, false, false, true>;
   }
   if (small)
     return staged ? (const void*)b128::ersd_cluster_kernel<DT, NR, AL, true, false> : (const void*)b128::ersd_cluster_kernel<DT, NR, AL, false, false>;
@@ -533,8 +535,8 @@ static const void* cluster_kernel(int cmax, bool staged, bool small, bool short_
   return (const void*)b256::ersd_cluster_kernel<DT, NR, AL, false, false>;
 }
 template <int DT, bool AL>
-static const void* cluster_kernel(int cmax, int roles, bool staged, bool small, bool short_way) {
-  return roles == 2 ? cluster_kernel<DT, AL, 2>(cmax, staged, small, short_way) : cluster_kernel<DT, AL, 1>(cmax, staged, small, short_way);
+static const void* cluster_kernel(bool verify, int cmax, int roles, bool staged, bool small, bool short_way) {
+  return roles == 2 ? cluster_kernel<DT, AL, 2>(verify, cmax, staged, small, short_way) : cluster_kernel<DT, AL, 1>(verify, cmax, staged, small, short_way);
 }
 
 // Whether a call can take a cluster kernel at all; cmax: most arrivals any of its races wants.
@@ -664,11 +666,12 @@ template <int DT, bool AL>
 static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeDesc& tree, int cmax, cudaStream_t st) {
   Params p = p_in;
   p.top_cmax = cmax;
-  int roles = (p.mode == kVerify && p.draft) ? 2 : 1;
+  const bool verify = p.mode == kVerify;
+  int roles = (verify && p.draft) ? 2 : 1;
   int CL = 1;
   const bool staged = cluster_staged(p, DT, roles, cmax);
   int lim = 8;
-  int ls = prepare_kernel(cluster_kernel<DT, AL>(cmax, roles, staged, false, false), kClusterSmemBytes, false, true, &lim);
+  int ls = prepare_kernel(cluster_kernel<DT, AL>(verify, cmax, roles, staged, false, false), kClusterSmemBytes, false, true, &lim);
   if (ls == ERSD_OK) ls = cluster_size(o, p, DT, cmax, staged, lim, &CL);
   if (ls != ERSD_OK) return ls;
   const int ntiles = (p.V + b256::kTile - 1) / b256::kTile;
@@ -687,7 +690,7 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
       split = true;
     }
     if (split) {
-      ls = prepare_kernel(cluster_kernel<DT, AL>(cmax, 1, staged, false, false), kClusterSmemBytes, false, true, &lim);
+      ls = prepare_kernel(cluster_kernel<DT, AL>(verify, cmax, 1, staged, false, false), kClusterSmemBytes, false, true, &lim);
       if (ls != ERSD_OK) return ls;
     }
     if (split && CL <= lim) {
@@ -727,7 +730,7 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
                    : roles == 2 ? DT == ERSD_BF16 && AL && blocks <= 3 * sm_count()
                                 : DT == ERSD_F32 && blocks > 3 * sm_count() && G > 16;
   if (short_way) {
-    ls = prepare_kernel(cluster_kernel<DT, AL>(cmax, roles, staged, small, true), kClusterSmemBytes, false, true, &lim);
+    ls = prepare_kernel(cluster_kernel<DT, AL>(verify, cmax, roles, staged, small, true), kClusterSmemBytes, false, true, &lim);
     if (ls != ERSD_OK) return ls;
     short_way = CL <= lim;
   }
@@ -735,7 +738,7 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
            cmax > 1 ? "ersd_cluster_top_kernel" : "ersd_cluster_kernel", DT == ERSD_BF16 ? "bf16" : "f32", roles,
            p.B * jobs, CL, threads, p.B * p.rows, staged ? "" : " (unstaged)",
            !short_way ? "" : cmax == 1 && !staged ? ", more tiles ahead" : ", short way");
-  const void* kernel = cluster_kernel<DT, AL>(cmax, roles, staged, small, short_way);
+  const void* kernel = cluster_kernel<DT, AL>(verify, cmax, roles, staged, small, short_way);
   if (small) {  // (the other builds are prepared by now)
     ls = prepare_kernel(kernel, staged ? kClusterSmemBytes : 0, false, false, nullptr);
     if (ls != ERSD_OK) return ls;
