@@ -728,7 +728,7 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
                    : staged     ? CL >= 4
                    : small      ? false
                    : roles == 2 ? DT == ERSD_BF16 && AL && blocks <= 3 * sm_count()
-                                : DT == ERSD_F32 && blocks > 3 * sm_count() && G > 16;
+                                : DT == ERSD_F32 && blocks > 3 * sm_count() && G >= 16;
   if (short_way) {
     ls = prepare_kernel(cluster_kernel<DT, AL>(verify, cmax, roles, staged, small, true), kClusterSmemBytes, false, true, &lim);
     if (ls != ERSD_OK) return ls;

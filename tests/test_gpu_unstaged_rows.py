@@ -53,10 +53,10 @@ def test_three_tiles_ahead(ersd, positions, V):  # noqa: F811
     check_verify(inp, out)
 
 
-@pytest.mark.parametrize("rows,V,more", [(100, 32000, False), (450, 34816, True), (450, 34817, True), (450, 32768, False), (300, 38912, False),
+@pytest.mark.parametrize("rows,V,more", [(100, 32000, False), (450, 34816, True), (450, 34817, True), (450, 32768, True), (450, 30720, False), (300, 38912, False),
                                          (150, 151936, True), (230, 69640, True)])
 def test_32_bit_rows_two_tiles_ahead(ersd, rows, V, more):  # noqa: F811
-    """One row per position: 17 tiles to a block and more, in more than three blocks to an SM."""
+    """One row per position: 16 tiles to a block and more, in more than three blocks to an SM."""
     logits = inputs(rows, 0, V, "f32")["target"]
     seeds = wl.make_seeds(7, V, rows)
     tok = torch.full((rows, 1, 1), -7, dtype=torch.int32, device="cuda")
