@@ -78,6 +78,20 @@ def test_several_arrivals_of_one_warp_and_of_one_thread(ersd, B, V, c, dtype):  
         check_sample(z, inp["seeds"], T, tok, key, c=c)
 
 
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("V", [900, 40000, 128256])
+def test_key_of_a_greedy_row_of_zeros(ersd, V, dtype):  # noqa: F811
+    """-z, without a sign, whether the row goes the short way or, all groups being tied, the long one."""
+    z = torch.zeros(2, 1, V, dtype=dtype, device="cuda")
+    z[1, 0, 5:] = -1.0
+    tok = torch.full((2, 1, 1), -7, dtype=torch.int32, device="cuda")
+    key = torch.full((2, 1, 1), -7.0, dtype=torch.float32, device="cuda")
+    ersd.ersd_race_sample(z, wl.make_seeds(3, 0, 2).cuda(), 0.0, tok, ersd.make_opts(out_key=key))
+    torch.cuda.synchronize()
+    assert "ersd_cluster_kernel" in ersd.ersd_last_launch()
+    assert (tok == 0).all() and (key.view(torch.int32) == 0).all()
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 def test_greedy_rows_among_others(ersd, dtype):  # noqa: F811
     """A call whose rows have temperatures of their own takes the short way's build, in which greedy rows go the long way."""
