@@ -112,6 +112,7 @@ struct Params {
   float* out_key;        // sample mode
   uint32_t* near_tie;    // count of races with two consecutive arrivals closer than 1e-5 (nullable)
   int extra;             // 1 when near-ties are counted: every race is run for one more arrival
+  int top_picks;         // its short way: groups a warp screens for races of three arrivals and more
   int top_cmax;          // cluster kernel for several arrivals: most arrivals any race of the call wants
   int top_split;         // the same kernel: 0, or 1 + the number of nodes with children when every row gets its own cluster
   int early;             // cluster kernels: let the next kernel on the stream start early
@@ -738,6 +739,7 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
            cmax > 1 ? "ersd_cluster_top_kernel" : "ersd_cluster_kernel", DT == ERSD_BF16 ? "bf16" : "f32", roles,
            p.B * jobs, CL, threads, p.B * p.rows, staged ? "" : " (unstaged)",
            !short_way ? "" : cmax == 1 && !staged ? ", more tiles ahead" : ", short way");
+  p.top_picks = CL * b256::kWarps >= 20 * cmax ? 4 : b256::kTopRounds;
   const void* kernel = cluster_kernel<DT, AL>(verify, cmax, roles, staged, small, short_way);
   if (small) {  // (the other builds are prepared by now)
     ls = prepare_kernel(kernel, staged ? kClusterSmemBytes : 0, false, false, nullptr);
