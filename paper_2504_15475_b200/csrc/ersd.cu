@@ -516,16 +516,20 @@ static int cluster_max_tiles(int dt, int roles, int cmax, bool aligned) {
 }
 
 // The build of the cluster kernels for rows of type DT, aligned (AL) or not, `roles` of them raced together.
-// short_way: the FAST builds of ersd_cluster_kernel, the DIRECT builds of ersd_cluster_top_kernel.
+// short_way: 0; 1 or 2: the FAST builds of ersd_cluster_kernel; the builds of ersd_cluster_top_kernel with the short way
+// (unstaged: with 1 or 2 tiles asked for ahead, 2 for aligned rows alone, and always for aligned bf16 ones).
 template <int DT, bool AL, int NR>
-static const void* cluster_kernel(bool verify, int cmax, bool staged, bool small, bool short_way) {
+static const void* cluster_kernel(bool verify, int cmax, bool staged, bool small, int short_way) {
   if (cmax > 1) {
     if constexpr (NR == 1) {
-      if (short_way)
-        return staged ? (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, true, true, true> : (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, false, true, true>;
-      if (!staged && !verify) return (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, false, false, false>;
+      if (short_way && staged) return (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, true, 1, true>;
+      if constexpr (AL)
+        if (short_way == 2 || (short_way && DT == ERSD_BF16)) return (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, false, 2, true>;
+      if constexpr (!AL || DT == ERSD_F32)
+        if (short_way) return (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, false, 1, true>;
+      if (!staged && !verify) return (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, false, 0, false>;
     }
-    return staged ? (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, true, false, true> : (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, false, false, true>;
+    return staged ? (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, true, 0, true> : (const void*)b256::ersd_cluster_top_kernel<DT, NR, AL, false, 0, true>;
   }
   if (small)
     return staged ? (const void*)b128::ersd_cluster_kernel<DT, NR, AL, true, false> : (const void*)b128::ersd_cluster_kernel<DT, NR, AL, false, false>;
@@ -536,7 +540,7 @@ static const void* cluster_kernel(bool verify, int cmax, bool staged, bool small
   return (const void*)b256::ersd_cluster_kernel<DT, NR, AL, false, false>;
 }
 template <int DT, bool AL>
-static const void* cluster_kernel(bool verify, int cmax, int roles, bool staged, bool small, bool short_way) {
+static const void* cluster_kernel(bool verify, int cmax, int roles, bool staged, bool small, int short_way) {
   return roles == 2 ? cluster_kernel<DT, AL, 2>(verify, cmax, staged, small, short_way) : cluster_kernel<DT, AL, 1>(verify, cmax, staged, small, short_way);
 }
 
@@ -672,7 +676,7 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   int CL = 1;
   const bool staged = cluster_staged(p, DT, roles, cmax);
   int lim = 8;
-  int ls = prepare_kernel(cluster_kernel<DT, AL>(verify, cmax, roles, staged, false, false), kClusterSmemBytes, false, true, &lim);
+  int ls = prepare_kernel(cluster_kernel<DT, AL>(verify, cmax, roles, staged, false, 0), kClusterSmemBytes, false, true, &lim);
   if (ls == ERSD_OK) ls = cluster_size(o, p, DT, cmax, staged, lim, &CL);
   if (ls != ERSD_OK) return ls;
   const int ntiles = (p.V + b256::kTile - 1) / b256::kTile;
@@ -691,7 +695,7 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
       split = true;
     }
     if (split) {
-      ls = prepare_kernel(cluster_kernel<DT, AL>(verify, cmax, 1, staged, false, false), kClusterSmemBytes, false, true, &lim);
+      ls = prepare_kernel(cluster_kernel<DT, AL>(verify, cmax, 1, staged, false, 0), kClusterSmemBytes, false, true, &lim);
       if (ls != ERSD_OK) return ls;
     }
     if (split && CL <= lim) {
@@ -725,15 +729,16 @@ static int launch_cluster_dt(const ersd_opts& o, const Params& p_in, const TreeD
   // Builds for some calls (where the device does not take them in clusters of this size: the general one).  Staged rows
   // in clusters of at least four blocks: the short way of ersd_cluster_kernel.  Unstaged rows, by blocks to an SM: see
   // cluster_ahead.  Several arrivals, with ten warps of the cluster to an arrival, unless all rows are greedy: see DIRECT.
-  bool short_way = cmax > 1     ? roles == 1 && CL * b256::kWarps >= 10 * cmax && (p.temps || p.T != 0.0f)
-                   : staged     ? CL >= 4
-                   : small      ? false
-                   : roles == 2 ? DT == ERSD_BF16 && AL && blocks <= 3 * sm_count()
-                                : DT == ERSD_F32 && blocks > 3 * sm_count() && G >= 16;
+  const int ahead = AL && (DT == ERSD_BF16 || G >= 16) ? 2 : 1;
+  int short_way = cmax > 1     ? (roles == 1 && CL * b256::kWarps >= 10 * cmax && (p.temps || p.T != 0.0f) ? ahead : 0)
+                  : staged     ? CL >= 4
+                  : small      ? 0
+                  : roles == 2 ? DT == ERSD_BF16 && AL && blocks <= 3 * sm_count()
+                               : DT == ERSD_F32 && blocks > 3 * sm_count() && G >= 16;
   if (short_way) {
-    ls = prepare_kernel(cluster_kernel<DT, AL>(verify, cmax, roles, staged, small, true), kClusterSmemBytes, false, true, &lim);
+    ls = prepare_kernel(cluster_kernel<DT, AL>(verify, cmax, roles, staged, small, short_way), kClusterSmemBytes, false, true, &lim);
     if (ls != ERSD_OK) return ls;
-    short_way = CL <= lim;
+    if (CL > lim) short_way = 0;
   }
   snprintf(g_last_launch, sizeof g_last_launch, "%s<%s, %d row(s) per cluster>: %d clusters of %d x %d threads, %d positions%s%s",
            cmax > 1 ? "ersd_cluster_top_kernel" : "ersd_cluster_kernel", DT == ERSD_BF16 ? "bf16" : "f32", roles,

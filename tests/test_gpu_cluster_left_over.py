@@ -52,7 +52,7 @@ def test_contenders_of_one_warp_and_of_one_thread(ersd, B, V, dtype):  # noqa: F
 
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("B,V,c", [(4, 131072, 2), (2, 100001, 4), (1, 131080, 8), (4, 128256, 12), (1, 40961, 5), (40, 70001, 4),
-                                   (30, 128256, 3), (30, 100001, 2)])
+                                   (30, 128256, 3), (30, 100001, 2), (36, 133000, 2)])
 def test_several_arrivals_of_one_warp_and_of_one_thread(ersd, B, V, c, dtype):  # noqa: F811
     """Staged and not; rows of ties, rows with fewer tokens than arrivals, infinities, and rows as drawn."""
     inp = inputs(2 * B, 0, V, "f32")
