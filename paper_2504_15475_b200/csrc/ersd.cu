@@ -408,7 +408,7 @@ static RaceKernel race_kernel(bool bf16, bool aligned, bool many, int threads) {
 //             the streaming kernel need about 180 KB);
 //   cluster:  the opt-in for clusters of 16 blocks; *limit = the largest cluster (a power of two) that it
 //             can be launched in: 16 where that is granted and such a cluster fits, else 8.
-// Done when a call first wants the kernel: asking for all 40 cluster builds at once was 3 of the 32 ms that a
+// Done when a call first wants the kernel: asking for all cluster builds (40 then) at once was 3 of the 32 ms that a
 // process's first call took (drafting 32.1 -> 29.4 ms, verification 33.6 -> 30.2; most of the rest is loading the code).
 struct KernelState {
   const void* kernel;
