@@ -9,18 +9,20 @@ import sys
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
-SRC = [os.path.join(HERE, "csrc", "ersd.cu"), os.path.join(HERE, "csrc", "ersd_tree.cpp")]
-DEPS = SRC + [os.path.join(HERE, "csrc", "ersd_math.cuh"), os.path.join(HERE, "csrc", "ersd_kernel.inc"), os.path.join(HERE, "csrc", "ersd_cluster.inc"), os.path.join(HERE, "csrc", "ersd_cluster_top.inc"), os.path.join(HERE, "csrc", "ersd_gsd.inc"), os.path.join(ROOT, "include", "ersd.h")]
+CSRC = os.path.join(HERE, "csrc")
+SRC = [os.path.join(CSRC, name) for name in ("ersd.cu", "ersd_cluster_bf16.cu", "ersd_cluster_f32.cu", "ersd_tree.cpp")]
+DEPS = SRC + [os.path.join(CSRC, name) for name in ("ersd_device.cuh", "ersd_math.cuh", "ersd_kernel.inc", "ersd_cluster.inc",
+                                                    "ersd_cluster_top.inc", "ersd_cluster_select.inc", "ersd_gsd.inc")]
+DEPS.append(os.path.join(ROOT, "include", "ersd.h"))
 LIB = os.path.join(HERE, "libersd.so")
 CALL_SRC = os.path.join(HERE, "csrc", "ersd_call.cpp")
 CALL_LIB = os.path.join(HERE, "_ersd_call.so")  # the calling side of binding.py
 
 
-def nvcc_command(out: str, extra=()):
+def nvcc_command(out: str, inputs, extra=()):
     # (--no-compress: unpacking the device code was half of the 28 ms that a process's first launch took; 13 without it)
     return ["nvcc", "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "--no-compress", "-std=c++17",
-            "--shared", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"),
-            "-I", os.path.join(HERE, "csrc"), *extra, "-o", out, *SRC]
+            "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC, *extra, "-o", out, *inputs]
 
 
 def call_command(out: str):
@@ -52,20 +54,33 @@ def _call_fresh() -> bool:
         return b"\0" + str(torch.__version__).encode() + b"\0" in f.read()
 
 
-def build(force: bool = False, verbose: bool = False) -> str:
-    jobs = []
-    if force or not _fresh(LIB, DEPS):
-        jobs.append((LIB, lambda out: nvcc_command(out, ("-Xptxas", "-v") if verbose else ())))
-    if force or not _call_fresh():
-        jobs.append((CALL_LIB, call_command))
-    running = []
-    for lib, command in jobs:
-        tmp = lib + ".tmp.%d" % os.getpid()
-        running.append((lib, tmp, subprocess.Popen(command(tmp))))
-    for lib, tmp, job in running:
+def _wait(jobs) -> None:
+    for what, job in jobs:
         if job.wait() != 0:
-            raise RuntimeError("building %s failed" % lib)
-        os.replace(tmp, lib)
+            raise RuntimeError("building %s failed" % what)
+
+
+def build(force: bool = False, verbose: bool = False) -> str:
+    tag = ".tmp.%d" % os.getpid()
+    running, objects = [], []
+    new_lib, new_call = force or not _fresh(LIB, DEPS), force or not _call_fresh()
+    if new_lib:
+        for src in SRC:
+            objects.append(os.path.join(HERE, os.path.basename(src) + tag + ".o"))
+            running.append((src, subprocess.Popen(nvcc_command(objects[-1], ["-c", src], ("-Xptxas", "-v") if verbose else ()))))
+    if new_call:
+        running.append((CALL_LIB, subprocess.Popen(call_command(CALL_LIB + tag))))
+    try:
+        _wait(running)
+        if new_lib:
+            _wait([(LIB, subprocess.Popen(nvcc_command(LIB + tag, ["--shared", *objects])))])
+            os.replace(LIB + tag, LIB)
+        if new_call:
+            os.replace(CALL_LIB + tag, CALL_LIB)
+    finally:
+        for path in objects:
+            if os.path.exists(path):
+                os.remove(path)
     return LIB
 
 
