@@ -55,9 +55,9 @@ def _call_fresh() -> bool:
 
 
 def _wait(jobs) -> None:
-    for what, job in jobs:
-        if job.wait() != 0:
-            raise RuntimeError("building %s failed" % what)
+    failed = [what for what, job in jobs if job.wait() != 0]  # (all have ended by then)
+    if failed:
+        raise RuntimeError("building %s failed" % ", ".join(failed))
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
