@@ -6,7 +6,7 @@ import torch
 from paper_2504_15475_b200 import workloads as wl
 
 from parity_util import check_sample, check_verify
-from test_gpu_unaligned_rows import ersd, inputs  # noqa: F401  (fixture)
+from test_gpu_unaligned_rows import ersd, guarded, inputs  # noqa: F401  (fixture)
 
 pytestmark = pytest.mark.gpu
 
@@ -39,11 +39,13 @@ def test_more_ties_than_a_warp_has_room_for(ersd, c, threads, split):  # noqa: F
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("V", [5000, 9003])
+@pytest.mark.parametrize("parent", [None, [-1, 0, 0, 0, 1, 1]])
 @pytest.mark.parametrize("threads", [128, 256])
-def test_ties_in_both_rows_of_a_node(ersd, threads, dtype):  # noqa: F811
-    """Trees of more than two rows per SM, aligned rows: ties in a node's target row, in its draft row, and in both."""
-    parent, B, V = [-1, 0, 0, 0, 1, 1], 80, 5000
-    inp = inputs(B, len(parent) - 1, V, "f32", parent=parent)
+def test_ties_in_both_rows_of_a_node(ersd, threads, parent, V, dtype):  # noqa: F811
+    """Chains, and trees of more than two rows per SM: ties in a node's target row, in its draft row, and in both."""
+    B, k = 80, 5
+    inp = inputs(B, k, V, "f32", parent=parent)
     inp["T"] = 0.0
     for b in range(0, B, 8):
         for name in ("target", "draft"):
@@ -54,7 +56,8 @@ def test_ties_in_both_rows_of_a_node(ersd, threads, dtype):  # noqa: F811
         inp["draft"][b + 5, :, 2:] = float("-inf")                            # fewer tokens than children
     for name in ("target", "draft"):
         inp[name] = wl._storage(inp[name], dtype)
-    out = ersd.verify(inp["target"].cuda(), inp["draft"].cuda(), inp["seeds"].cuda(), 0.0, want_rows=True, parent=parent,
+    on_device = guarded if V % 8 else torch.Tensor.cuda
+    out = ersd.verify(on_device(inp["target"]), on_device(inp["draft"]), inp["seeds"].cuda(), 0.0, want_rows=True, parent=parent,
                       kernel_path=1, block_threads=threads)
     torch.cuda.synchronize()
     assert "ersd_race_kernel" in ersd.ersd_last_launch() and "pooled" not in ersd.ersd_last_launch()
